@@ -107,11 +107,15 @@ int ax_elems_per_block(int p, bool fp32) {
   const int N = p + 1;
   const int t = tile_get(p, fp32).ax_ne;
   if (t >= 1 && t * N * N <= 512) return t;
-  // FP64 even N (the folded kernel): measured on GB300 at 32^3 elements, elements per block
-  // N = 4: 8 (16: 0.144 -> 0.138 ms), N = 6: 8 (7: 0.543 -> 0.525 ms), N = 10: 3 (2: 3.38 ->
-  // 3.26 ms); N = 8 keeps 4 (1 to 4 within 0.5%)
-  if (!fp32 && (N == 4 || N == 6)) return 8;
-  if (!fp32 && N == 10) return 3;
+  // FP64 (ax_fx_kernel), measured on GB300 (us per launch by elements per block): N = 4, 32^3:
+  // 2 54, 4 55, 8 57, 12 62; N = 5, 24^3: 2 62, 4 63, 10 59; N = 6, 32^3: 2 225, 4 203, 7 190;
+  // N = 7, 24^3: 1 154, 3 147, 5 142; N = 8, 32^3: 1 419, 2 406, 3 434, 4 446; N = 9, 20^3: 1 196,
+  // 2 213, 3 197; N = 10, 20^3: 1 290, 2 269; N = 11, 16^3: 1 197, 2 230.  Whole warps of lines
+  // and several small blocks per SM, which hide each other's barriers
+  if (!fp32) {
+    constexpr int ne64[SE_MAX_ORDER + 2] = {0, 0, 32, 14, 4, 10, 7, 5, 2, 3, 2, 1};
+    return ne64[N];
+  }
   const int ne = 256 / (N * N);
   return ne < 1 ? 1 : ne;
 }
@@ -165,15 +169,9 @@ static int ax_local_generic_df(const Level& lv, const double* u, double* y, cons
 
 template <class T>
 int ax_local(const Level& lv, const T* u, T* y, bool mask_in, cudaStream_t s, const T* sub) {
-  const T* G;
-  const T* D;
-  if constexpr (sizeof(T) == 8) {
-    G = lv.G64;
-    D = lv.D64;
-  } else {
-    G = lv.G32;
-    D = lv.D32;
-  }
+  const void* G;
+  if constexpr (sizeof(T) == 8) G = lv.G64;
+  else G = lv.G32;
   SE_CHECK(G != nullptr, SE_EINVAL, "ax_local: geometric factors for this precision missing");
   const int N = lv.N;
   const double pts = (double)lv.L;
@@ -188,20 +186,17 @@ int ax_local(const Level& lv, const T* u, T* y, bool mask_in, cudaStream_t s, co
       if (ax_eo_supported(lv.p)) return ax_local_eo_df(lv, u, y, s, sub);
       return ax_local_generic_df(lv, u, y, sub, s);
     }
-    if (!mask_in && ax_eo_supported(lv.p) && lv.eo64) return ax_local_eo(lv, u, y, s, sub);
+    return ax_local_fx(lv, u, y, mask_in, sub, nullptr, ax_elems_per_block(lv.p, false), false, s);
   }
-  switch (N) {
-    case 2: return launch_ax<2, T>(lv, u, y, G, D, mask_in, sub, s);
-    case 3: return launch_ax<3, T>(lv, u, y, G, D, mask_in, sub, s);
-    case 4: return launch_ax<4, T>(lv, u, y, G, D, mask_in, sub, s);
-    case 5: return launch_ax<5, T>(lv, u, y, G, D, mask_in, sub, s);
-    case 6: return launch_ax<6, T>(lv, u, y, G, D, mask_in, sub, s);
-    case 7: return launch_ax<7, T>(lv, u, y, G, D, mask_in, sub, s);
-    case 8: return launch_ax<8, T>(lv, u, y, G, D, mask_in, sub, s);
-    case 9: return launch_ax<9, T>(lv, u, y, G, D, mask_in, sub, s);
-    case 10: return launch_ax<10, T>(lv, u, y, G, D, mask_in, sub, s);
-    case 11: return launch_ax<11, T>(lv, u, y, G, D, mask_in, sub, s);
-    default: set_error("ax_local: unsupported N=%d", N); return SE_EINVAL;
+  if constexpr (sizeof(T) == 4) {
+    switch (N) {
+#define SE_AX_CASE(NN) \
+  case NN: return launch_ax<NN, T>(lv, u, y, lv.G32, lv.D32, mask_in, sub, s);
+      SE_AX_CASE(2) SE_AX_CASE(3) SE_AX_CASE(4) SE_AX_CASE(5) SE_AX_CASE(6)
+      SE_AX_CASE(7) SE_AX_CASE(8) SE_AX_CASE(9) SE_AX_CASE(10) SE_AX_CASE(11)
+#undef SE_AX_CASE
+      default: set_error("ax_local: unsupported N=%d", N); return SE_EINVAL;
+    }
   }
 }
 
@@ -488,15 +483,14 @@ int gs_apply(const Level& lv, T* u, bool mask, cudaStream_t s) {
 }
 
 // ------------------------------------------------------------------ folded FP64 operator
-// The even-odd kernel sums the x-interfaces inside its blocks and masks (ax_local_eo_fold); the
+// The operator kernel sums the x-interfaces inside its blocks and masks (ax_local_fx, fold); the
 // x-interfaces between blocks follow (gs_fold_fixup), then the fused y/z launch, so the x direction
 // is complete before y and z start, as in the sweeps above, and every copy of a node gets the
 // same bits.  This removes the x sweep, which
 // reads and writes every sector of the vector (an x-interface copy is the first or last value of
 // a row of N), from the operator applications of the solve.
 bool ax_fold_ok(const Level& lv) {
-  return !ax_df_route(lv) && lv.eo64 && ax_eo_supported(lv.p) && !lv.gsm_ids && lv.nel[0] >= 1 &&
-         lv.nel[1] >= 1 && lv.nel[2] >= 1;
+  return !ax_df_route(lv) && !lv.gsm_ids && lv.nel[0] >= 1 && lv.nel[1] >= 1 && lv.nel[2] >= 1;
 }
 
 template <int N>
@@ -517,7 +511,7 @@ static int gs_after_fold(const Level& lv, double* y, int NE, cudaStream_t s) {
 }
 
 int ax_apply_folded(const Level& lv, const double* u, double* y, const double* b, cudaStream_t s,
-                    const double* dinv) {
+                    const double* dinv, bool mask_in) {
   const int NE = ax_elems_per_block(lv.p, false);
   {
     const double pts = (double)lv.L;
@@ -526,14 +520,14 @@ int ax_apply_folded(const Level& lv, const double* u, double* y, const double* b
     ProfScope prof(SE_K_AX, s, pts,
                    pts * (8.0 + (b ? 1.0 : 0.0) + (dinv ? 1.0 : 0.0)) * sizeof(double),
                    pts * (12.0 * lv.N + 15.0), prof_variant<double>(lv.p));
-    SE_TRY(ax_local_eo_fold(lv, u, y, b, NE, s, dinv));
+    SE_TRY(ax_local_fx(lv, u, y, mask_in, b, dinv, NE, true, s));
   }
   switch (lv.N) {
-    case 2: return gs_after_fold<2>(lv, y, NE, s);
-    case 4: return gs_after_fold<4>(lv, y, NE, s);
-    case 6: return gs_after_fold<6>(lv, y, NE, s);
-    case 8: return gs_after_fold<8>(lv, y, NE, s);
-    case 10: return gs_after_fold<10>(lv, y, NE, s);
+#define SE_FOLD_CASE(NN) \
+  case NN: return gs_after_fold<NN>(lv, y, NE, s);
+    SE_FOLD_CASE(2) SE_FOLD_CASE(3) SE_FOLD_CASE(4) SE_FOLD_CASE(5) SE_FOLD_CASE(6)
+    SE_FOLD_CASE(7) SE_FOLD_CASE(8) SE_FOLD_CASE(9) SE_FOLD_CASE(10) SE_FOLD_CASE(11)
+#undef SE_FOLD_CASE
     default: set_error("ax_apply_folded: unsupported N=%d", lv.N); return SE_EINVAL;
   }
 }
@@ -592,6 +586,7 @@ int se_ax(se_mesh_t m, const double* u, double* y, int flags, void* stream) {
     if (mask) return apply_mask64(lv, y, s);
     return SE_OK;
   }
+  if (assemble && mask && ax_fold_ok(lv)) return ax_apply_folded(lv, u, y, nullptr, s, nullptr, true);
   SE_TRY(ax_local<double>(lv, u, y, mask, s));
   if (assemble) return gs_apply<double>(lv, y, mask, s);
   if (mask) return apply_mask64(lv, y, s);

@@ -87,23 +87,13 @@ __device__ __forceinline__ void eo_apply(const T* __restrict__ Ep, const T* __re
 }
 
 // tables: [0] Ep(D), [1] Om(D), [2] Ep(D^T), [3] Om(D^T), each H*H
-// FOLD (T = double): the block's elements are consecutive in the element numbering, so
-// neighbours along x (same row of the lattice, nx elements per row) are usually in the same
-// block.  The kernel then also does the x part of QQ^T for them: both copies of each such
-// x-interface node get left + right (the same bits on both sides), and it applies the Dirichlet
-// mask (bit f of `bits`: face f = x0, x1, y0, y1, z0, z1 is Dirichlet); the x-interfaces between
-// consecutive blocks are left to gs_fold_fixup_x.
-// SCALE (with FOLD): the input is dinv .* u, formed as it is loaded (the first step of a
-// Jacobi-Chebyshev smoother applies A to D^-1 r without storing D^-1 r).
-template <int N, typename T, bool FOLD = false, bool SCALE = false>
+template <int N, typename T>
 __global__ void __launch_bounds__(512) ax_eo_kernel(int64_t E, int NE, const double* __restrict__ u,
                                                     const T* __restrict__ G, int64_t L,
                                                     const T* __restrict__ tables,
                                                     double* __restrict__ y,
                                                     const uint8_t* __restrict__ pflag,
-                                                    const double* __restrict__ sub, int nx = 0,
-                                                    int ny = 0, int nz = 0, int bits = 0,
-                                                    const double* __restrict__ dinv = nullptr) {
+                                                    const double* __restrict__ sub) {
   constexpr int N2 = N * N, N3 = N * N * N, H = N / 2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* tab = reinterpret_cast<T*>(smem_raw);                    // 4 H^2
@@ -120,10 +110,7 @@ __global__ void __launch_bounds__(512) ax_eo_kernel(int64_t E, int NE, const dou
   const int64_t eb = e * N3;
   if (valid) {
 #pragma unroll
-    for (int q = 0; q < N; ++q) {
-      if constexpr (SCALE) su[t + N2 * q] = u[eb + t + N2 * q] * dinv[eb + t + N2 * q];
-      else su[t + N2 * q] = from_io<T>(u[eb + t + N2 * q]);
-    }
+    for (int q = 0; q < N; ++q) su[t + N2 * q] = from_io<T>(u[eb + t + N2 * q]);
   }
   __syncthreads();
   const T* EpD = tab;
@@ -159,110 +146,11 @@ __global__ void __launch_bounds__(512) ax_eo_kernel(int64_t E, int NE, const dou
   __syncthreads();
   if (valid) eo_apply<N, true>(EpT, OmT, st, sy, a + N * b, N2);
   __syncthreads();
-  if constexpr (FOLD) {
-    static_assert(sizeof(T) == sizeof(double), "the folded output is FP64");
-    // the kernel is bound by the FP64 pipe, where a warp instruction costs the same with 2 or 32
-    // lanes active: each interface pair is added once, by one lane of densely packed warps, and
-    // the weights 2^-(interfaces) of the residual form are built from their exponent bits
-    double* so0 = reinterpret_cast<double*>(tab + 4 * H * H);  // element 0 of the block
-    double* so = reinterpret_cast<double*>(sy);
-    // thread (le, t = i + N j) holds the points (i, j, k) of its element, k = 0..N-1; its place
-    // in the lattice gives the multiplicity (a copy on an interior interface normal to a
-    // direction has 2 copies along it) and the Dirichlet mask
-    const int i = t % N, j = t / N;
-    const int ei = (int)e;  // E < 2^31
-    const int ex = ei % nx, ey = (ei / nx) % ny, ez = ei / (nx * ny);
-    if (sub) {  // residual form: each copy's b / multiplicity - (A_L u), in place
-      if (valid) {
-        const int xy = (int)((i == 0 && ex > 0) || (i == N - 1 && ex < nx - 1)) +
-                       (int)((j == 0 && ey > 0) || (j == N - 1 && ey < ny - 1));
+  if (valid) {
 #pragma unroll
-        for (int q = 0; q < N; ++q) {
-          const int pt = t + N2 * q;
-          const int zin = (int)((q == 0 && ez > 0) || (q == N - 1 && ez < nz - 1));
-          const double w = __longlong_as_double((long long)(1023 - xy - zin) << 52);
-          so[pt] = sub[eb + pt] * w - so[pt];
-        }
-      }
-      __syncthreads();
-    }
-    // x-interfaces inside the block: (N - 1, j, k) of element lp and (0, j, k) of lp + 1 when
-    // both lie in one row; both copies get left + right
-    const int64_t e0 = (int64_t)blockIdx.x * NE;
-    for (int idx = threadIdx.x; idx < (NE - 1) * N2; idx += blockDim.x) {
-      const int lp = idx / N2, jk = idx - lp * N2;
-      const int el = (int)(e0 + lp);
-      if (el + 1 < E && el % nx < nx - 1) {
-        double* a = so0 + lp * 4 * N3 + (N - 1) + N * jk;
-        double* b = a + 4 * N3 - (N - 1);
-        const double v = *a + *b;
-        *a = v;
-        *b = v;
-      }
-    }
-    __syncthreads();
-    if (valid) {
-      const bool dxy = ((bits & 1) && i == 0 && ex == 0) || ((bits & 2) && i == N - 1 && ex == nx - 1) ||
-                       ((bits & 4) && j == 0 && ey == 0) || ((bits & 8) && j == N - 1 && ey == ny - 1);
-#pragma unroll
-      for (int q = 0; q < N; ++q) {
-        const bool dz = ((bits & 16) && q == 0 && ez == 0) || ((bits & 32) && q == N - 1 && ez == nz - 1);
-        y[eb + t + N2 * q] = (dxy || dz) ? 0.0 : so[t + N2 * q];
-      }
-    }
-  } else {
-    if (valid) {
-#pragma unroll
-      for (int q = 0; q < N; ++q)
-        y[eb + t + N2 * q] = ax_output(io_cast<double>(sy[t + N2 * q]), sub, pflag, eb + t + N2 * q);
-    }
+    for (int q = 0; q < N; ++q)
+      y[eb + t + N2 * q] = ax_output(io_cast<double>(sy[t + N2 * q]), sub, pflag, eb + t + N2 * q);
   }
-}
-
-// The x-interfaces that ax_eo_kernel<FOLD> leaves: element e = (b + 1) NE - 1, the last of block b,
-// and e + 1, the first of block b + 1, when both lie in one row.  Thread: (boundary, point (j, k)
-// of the face).  Masked copies are zero on both sides (a node's copies are all masked or none).
-template <int N>
-__global__ void gs_fold_fixup_x(int64_t E, int NE, int nx, double* __restrict__ y) {
-  constexpr int N2 = N * N, N3 = N2 * N;
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t nbnd = (E + NE - 1) / NE - 1;
-  if (t >= nbnd * N2) return;
-  const int64_t b = t / N2;
-  const int jk = (int)(t - b * N2);
-  const int64_t e = (b + 1) * NE - 1;
-  if (e + 1 >= E || (int)(e % nx) == nx - 1) return;
-  const int64_t ia = e * N3 + (N - 1) + (int64_t)N * jk;  // (N - 1, j, k) of e
-  const int64_t ib = (e + 1) * N3 + (int64_t)N * jk;      // (0, j, k) of e + 1
-  const double v = y[ia] + y[ib];
-  y[ia] = v;
-  y[ib] = v;
-}
-
-template <int N, bool SCALE>
-static int launch_ax_eo_fold_t(const Level& lv, const double* u, double* y, const double* sub, int NE,
-                               const double* dinv, cudaStream_t s) {
-  constexpr int H = N / 2;
-  const int threads = NE * N * N;
-  const size_t smem = (4 * H * H + (size_t)NE * 4 * N * N * N) * sizeof(double);
-  static const cudaError_t attr = cudaFuncSetAttribute(
-      ax_eo_kernel<N, double, true, SCALE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-  SE_CUDA(attr);
-  const unsigned blocks = (unsigned)((lv.E + NE - 1) / NE);
-  int bits = 0;
-  for (int f = 0; f < 6; ++f)
-    if (lv.bc[f] == SE_BC_DIRICHLET) bits |= 1 << f;
-  ax_eo_kernel<N, double, true, SCALE><<<blocks, threads, smem, s>>>(
-      lv.E, NE, u, lv.G64, lv.L, lv.eo64, y, lv.pflag, sub, lv.nel[0], lv.nel[1], lv.nel[2], bits, dinv);
-  SE_LAUNCH_CHECK();
-  return SE_OK;
-}
-
-template <int N>
-static int launch_ax_eo_fold(const Level& lv, const double* u, double* y, const double* sub, int NE,
-                             cudaStream_t s, const double* dinv) {
-  return dinv ? launch_ax_eo_fold_t<N, true>(lv, u, y, sub, NE, dinv, s)
-              : launch_ax_eo_fold_t<N, false>(lv, u, y, sub, NE, nullptr, s);
 }
 
 template <int N, typename T>
@@ -306,41 +194,6 @@ static int ax_eo_dispatch(const Level& lv, const double* u, double* y, const T* 
     case 10: return launch_ax_eo<10, T>(lv, u, y, G, tab, sub, s);
     default: set_error("ax_eo: unsupported N=%d", lv.N); return SE_EINVAL;
   }
-}
-
-int ax_local_eo(const Level& lv, const double* u, double* y, cudaStream_t s, const double* sub) {
-  SE_CHECK(lv.eo64 != nullptr, SE_EINVAL, "ax_eo: folded tables missing");
-  return ax_eo_dispatch<double>(lv, u, y, lv.G64, lv.eo64, s, sub);
-}
-
-int ax_local_eo_fold(const Level& lv, const double* u, double* y, const double* sub, int NE,
-                     cudaStream_t s, const double* dinv) {
-  SE_CHECK(lv.eo64 != nullptr && lv.nel[0] >= 1, SE_EINVAL, "ax_eo_fold: folded tables or lattice missing");
-  switch (lv.N) {
-    case 2: return launch_ax_eo_fold<2>(lv, u, y, sub, NE, s, dinv);
-    case 4: return launch_ax_eo_fold<4>(lv, u, y, sub, NE, s, dinv);
-    case 6: return launch_ax_eo_fold<6>(lv, u, y, sub, NE, s, dinv);
-    case 8: return launch_ax_eo_fold<8>(lv, u, y, sub, NE, s, dinv);
-    case 10: return launch_ax_eo_fold<10>(lv, u, y, sub, NE, s, dinv);
-    default: set_error("ax_eo_fold: unsupported N=%d", lv.N); return SE_EINVAL;
-  }
-}
-
-int gs_fold_fixup(const Level& lv, double* y, int NE, cudaStream_t s) {
-  const int64_t nbnd = (lv.E + NE - 1) / NE - 1;
-  if (nbnd <= 0 || lv.nel[0] <= 1) return SE_OK;
-  const int64_t n = nbnd * lv.N * lv.N;
-  switch (lv.N) {
-#define SE_FIX_CASE(NN)                                                                      \
-  case NN:                                                                                   \
-    gs_fold_fixup_x<NN><<<grid_for(n, 256), 256, 0, s>>>(lv.E, NE, lv.nel[0], y);            \
-    break;
-    SE_FIX_CASE(2) SE_FIX_CASE(4) SE_FIX_CASE(6) SE_FIX_CASE(8) SE_FIX_CASE(10)
-#undef SE_FIX_CASE
-    default: set_error("gs_fold_fixup: unsupported N=%d", lv.N); return SE_EINVAL;
-  }
-  SE_LAUNCH_CHECK();
-  return SE_OK;
 }
 
 int ax_local_eo_df(const Level& lv, const double* u, double* y, cudaStream_t s, const double* sub) {

@@ -1,0 +1,402 @@
+// FP64 local Ax with folded line contractions in block floating point (fxp.h), every N.
+//
+// Sum factorisation: (ur, us, ut) = (D_r u, D_s u, D_t u);  w = G (ur, us, ut);
+// y = D_r^T wr + D_s^T ws + D_t^T wt.  The six contractions run on the integer pipe: u is split
+// once into fixed point on the scale of the element's largest value, the gradients come back as
+// doubles for the pointwise product with G (9 FP64 instructions per point, what is left on the
+// FP64 pipe), w is split again on its own scale, and the three parts of y are added as 64-bit
+// integers before the one rounding to double.  The derivative matrix is centro-antisymmetric, so
+// a line of N values costs N^2/2 terms.
+//
+// NE elements per block, N^2 threads per element; each thread owns one line per direction.  Per
+// element three arrays U, R, S in shared memory (rows of N padded to an odd stride, so that lines
+// along every direction are read without bank conflicts), each updated in place: a thread
+// writes a line's results over the line, and the column (i, j, 0..N-1) it owns holds wt in U.
+//
+// FOLD: the block's elements are consecutive in the element numbering, so neighbours along x
+// (same row of the lattice, nx elements per row) are usually in the same block.  The kernel then
+// also does the x part of QQ^T for them: both copies of each such x-interface node get
+// left + right (the same bits on both sides), and it applies the Dirichlet mask (bit f of `bits`:
+// face f = x0, x1, y0, y1, z0, z1 is Dirichlet); the x-interfaces between consecutive blocks are
+// left to gs_fold_fixup_x.
+//
+// Measured on GB300 (us per launch; in brackets the even-odd FP64 kernel this one replaced, which ran at
+// the FP64 pipe's 2 FMA/clk/SM): 32^3 elements p = 7 417 [1420], p = 5 187 [525], p = 3 56 [138]; even
+// orders (unfolded in FP64) 20^3 p = 8 202 [725].  Memory needs 158 us of the 417, the 9 FP64
+// instructions per point 240, and the integer pipes about the same: what is left are the waits between
+// them, so resident warps count (64 registers: 417, 80: 440, 128: 485; before the conversions back
+// were branch-free and G was prefetched to L2, 530 to 560).
+//
+// Elements whose values cannot share a scale (infinities, NaN, magnitudes at the ends of the
+// range) send their block to ax_slow_block, the same operator in FP64.
+#include "fxp.h"
+#include "se_internal.h"
+
+namespace se {
+
+struct AxFxArgs {
+  int64_t E, L;
+  int NE;
+  const double *u, *G, *D, *sub, *dinv;
+  const uint8_t* pflag;
+  double* y;
+  int mask_in;             // zero the Dirichlet values of u as they are read
+  int nx, ny, nz, bits;    // FOLD
+};
+
+template <int N>
+struct AxFxDims {
+  static constexpr int NP = N % 2 ? N : N + 1;     // padded row: odd, so 8-byte lines do not conflict
+  static constexpr int PLANE = NP * N, VOL = NP * N * N;
+};
+
+// Input value of a local point: u, or D^-1 u, zero on masked points.
+__device__ __forceinline__ double ax_fx_input(const AxFxArgs& a, int64_t gi, bool zero) {
+  double v = a.u[gi];
+  if (a.dinv) v *= a.dinv[gi];
+  return zero ? 0.0 : v;
+}
+
+// A_L u of the block's elements in FP64, columns of results to U (the caller's column of each
+// thread).  Every thread of the block calls it.
+template <int N>
+__device__ __noinline__ void ax_slow_block(const AxFxArgs& a, int64_t e, bool valid, int i, int j, unsigned zmask,
+                                           double* U, double* R, double* S) {
+  constexpr int N2 = N * N, NP = AxFxDims<N>::NP, PL = AxFxDims<N>::PLANE;
+  const int64_t eb = e * (N2 * N) + i + N * j;
+  double* Uc = U + i + NP * j;
+  __syncthreads();
+  if (valid) {
+#pragma unroll 1
+    for (int k = 0; k < N; ++k) Uc[PL * k] = ax_fx_input(a, eb + N2 * k, (zmask >> k) & 1u);
+  }
+  __syncthreads();
+  double ry[N];
+#pragma unroll
+  for (int l = 0; l < N; ++l) ry[l] = 0.0;
+  if (valid) {
+#pragma unroll 1
+    for (int k = 0; k < N; ++k) {
+      double ur = 0.0, us = 0.0, ut = 0.0;
+#pragma unroll 1
+      for (int l = 0; l < N; ++l) {
+        ur = fma(a.D[i * N + l], U[l + NP * j + PL * k], ur);
+        us = fma(a.D[j * N + l], U[i + NP * l + PL * k], us);
+        ut = fma(a.D[k * N + l], Uc[PL * l], ut);
+      }
+      const double* g = a.G + eb + N2 * k;
+      const double grr = g[0], grs = g[a.L], grt = g[2 * a.L], gss = g[3 * a.L], gst = g[4 * a.L], gtt = g[5 * a.L];
+      R[i + NP * j + PL * k] = fma(grt, ut, fma(grs, us, grr * ur));
+      S[i + NP * j + PL * k] = fma(gst, ut, fma(gss, us, grs * ur));
+      const double wt = fma(gtt, ut, fma(gst, us, grt * ur));
+#pragma unroll
+      for (int l = 0; l < N; ++l) ry[l] = fma(a.D[k * N + l], wt, ry[l]);
+    }
+  }
+  __syncthreads();
+  if (valid) {
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      double acc = ry[k];
+#pragma unroll 1
+      for (int l = 0; l < N; ++l) {
+        acc = fma(a.D[l * N + i], R[l + NP * j + PL * k], acc);
+        acc = fma(a.D[l * N + j], S[i + NP * l + PL * k], acc);
+      }
+      Uc[PL * k] = acc;
+    }
+  }
+}
+
+// Registers: the kernel waits on memory, shared memory and dependent integer operations in turn, so
+// resident warps are worth more than registers up to the point where lines spill.
+template <int N>
+constexpr int ax_fx_regs() { return N <= 8 ? 64 : (N <= 10 ? 72 : 96); }
+
+template <int N, bool FOLD>
+__global__ void __maxnreg__(ax_fx_regs<N>())
+    ax_fx_kernel(const __grid_constant__ AxFxArgs a, const __grid_constant__ FxFold<N, N> tD,
+                 const __grid_constant__ FxFold<N, N> tT) {
+  constexpr int N2 = N * N, N3 = N2 * N, NP = AxFxDims<N>::NP, PL = AxFxDims<N>::PLANE, VOL = AxFxDims<N>::VOL;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int le = threadIdx.x / N2;
+  const int t = threadIdx.x - le * N2;
+  const int i = t % N, j = t / N;  // the thread's column; also (j, k) of its r-line, (i, k) of its s-line
+  double* U = reinterpret_cast<double*>(smem_raw) + (size_t)le * 3 * VOL;
+  double* R = U + VOL;
+  double* S = R + VOL;
+  unsigned* mags = reinterpret_cast<unsigned*>(reinterpret_cast<double*>(smem_raw) + (size_t)a.NE * 3 * VOL);
+  const int64_t e = (int64_t)blockIdx.x * a.NE + le;
+  const bool valid = e < a.E;
+  const int64_t eb = e * N3 + t;
+  const int col = i + NP * j, rl = NP * i + PL * j, sl = i + PL * j;  // lines: column, (j=i,k=j), (i,k=j)
+  if (t == 0) mags[2 * le] = mags[2 * le + 1] = 0u;
+  // the geometric factors are needed after the forward contractions: on their way to L2 meanwhile
+  if (valid && t < 6 && N2 >= 6) fx_prefetch(a.G + t * a.L + e * N3, N3);
+  // Dirichlet points of the column (bit k)
+  unsigned zmask = 0u;
+  int ex = 0, ey = 0, ez = 0;
+  if constexpr (FOLD) {
+    const int ei = (int)e;  // E < 2^31
+    ex = ei % a.nx;
+    ey = (ei / a.nx) % a.ny;
+    ez = ei / (a.nx * a.ny);
+    const bool dxy = ((a.bits & 1) && i == 0 && ex == 0) || ((a.bits & 2) && i == N - 1 && ex == a.nx - 1) ||
+                     ((a.bits & 4) && j == 0 && ey == 0) || ((a.bits & 8) && j == N - 1 && ey == a.ny - 1);
+    if (dxy) zmask = (1u << N) - 1u;
+    if ((a.bits & 16) && ez == 0) zmask |= 1u;
+    if ((a.bits & 32) && ez == a.nz - 1) zmask |= 1u << (N - 1);
+  } else if (a.mask_in && valid) {
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+      if (!(a.pflag[eb + N2 * k] & PF_FREE)) zmask |= 1u << k;
+  }
+  const unsigned zin = a.mask_in ? zmask : 0u;
+  __syncthreads();
+  bool bad = false;
+  {
+    double v[N];
+    unsigned mag = 0u;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      v[k] = valid ? ax_fx_input(a, eb + N2 * k, (zin >> k) & 1u) : 0.0;
+      mag = max(mag, fx_mag(v[k]));
+    }
+    if (mag) atomicMax(&mags[2 * le], mag);
+    __syncthreads();
+    mag = mags[2 * le];
+    bad = fx_bad(mag);
+    const int E = fx_exponent(mag);
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      int h, l;
+      fx_split(v[k], E, h, l);
+      reinterpret_cast<int2*>(U)[col + PL * k] = make_int2(h, l);
+    }
+  }
+  bad = __syncthreads_or(bad);
+  if (!bad) {
+    const int eb1 = fx_exponent(mags[2 * le]) - tD.k;
+    {
+      int h[N], l[N];
+#pragma unroll
+      for (int q = 0; q < N; ++q) {
+        const int2 x = reinterpret_cast<const int2*>(U)[rl + q];
+        h[q] = x.x;
+        l[q] = x.y;
+      }
+      fx_contract<N, N, -1>(tD, h, l, [&](int q, long long r) { R[rl + q] = fx_double(r, eb1); });
+#pragma unroll
+      for (int q = 0; q < N; ++q) {
+        const int2 x = reinterpret_cast<const int2*>(U)[sl + NP * q];
+        h[q] = x.x;
+        l[q] = x.y;
+      }
+      fx_contract<N, N, -1>(tD, h, l, [&](int q, long long r) { S[sl + NP * q] = fx_double(r, eb1); });
+    }
+    __syncthreads();
+    // t-lines and the pointwise factors: the thread's column
+    {
+      int h[N], l[N];
+#pragma unroll
+      for (int q = 0; q < N; ++q) {
+        const int2 x = reinterpret_cast<const int2*>(U)[col + PL * q];
+        h[q] = x.x;
+        l[q] = x.y;
+      }
+      unsigned mag = 0u;
+      fx_contract<N, N, -1>(tD, h, l, [&](int q, long long r) {
+        const double ut = fx_double(r, eb1), ur = R[col + PL * q], us = S[col + PL * q];
+        double grr = 0.0, grs = 0.0, grt = 0.0, gss = 0.0, gst = 0.0, gtt = 0.0;
+        if (valid) {
+          const double* g = a.G + eb + N2 * q;
+          grr = g[0], grs = g[a.L], grt = g[2 * a.L], gss = g[3 * a.L], gst = g[4 * a.L], gtt = g[5 * a.L];
+        }
+        const double wr = fma(grt, ut, fma(grs, us, grr * ur));
+        const double ws = fma(gst, ut, fma(gss, us, grs * ur));
+        const double wt = fma(gtt, ut, fma(gst, us, grt * ur));
+        R[col + PL * q] = wr;
+        S[col + PL * q] = ws;
+        U[col + PL * q] = wt;
+        mag = max(max(mag, fx_mag(wr)), max(fx_mag(ws), fx_mag(wt)));
+      });
+      if (mag) atomicMax(&mags[2 * le + 1], mag);
+    }
+    __syncthreads();
+    const unsigned mag2 = mags[2 * le + 1];
+    const int E2 = fx_exponent(mag2);
+    {
+      int h[N], l[N];
+#pragma unroll
+      for (int q = 0; q < N; ++q) fx_split(R[rl + q], E2, h[q], l[q]);
+      fx_contract<N, N, -1>(tT, h, l, [&](int q, long long r) { reinterpret_cast<long long*>(R)[rl + q] = r; });
+#pragma unroll
+      for (int q = 0; q < N; ++q) fx_split(S[sl + NP * q], E2, h[q], l[q]);
+      fx_contract<N, N, -1>(tT, h, l, [&](int q, long long r) { reinterpret_cast<long long*>(S)[sl + NP * q] = r; });
+    }
+    bad = __syncthreads_or(fx_bad(mag2));
+    if (!bad) {
+      const int eb2 = E2 - tT.k;
+      int h[N], l[N];
+#pragma unroll
+      for (int q = 0; q < N; ++q) fx_split(U[col + PL * q], E2, h[q], l[q]);
+      fx_contract<N, N, -1>(tT, h, l, [&](int q, long long r) {
+        r += reinterpret_cast<const long long*>(R)[col + PL * q] + reinterpret_cast<const long long*>(S)[col + PL * q];
+        U[col + PL * q] = fx_double(r, eb2);
+      });
+    }
+  }
+  if (bad) ax_slow_block<N>(a, e, valid, i, j, zin, U, R, S);
+  // U: A_L u, each thread's own column
+  if constexpr (FOLD) {
+    // residual form: each copy's b / multiplicity - (A_L u); a copy on an interior interface
+    // normal to a direction has 2 copies along it, so the weight is a power of two, built from its
+    // exponent bits
+    double yv[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) yv[k] = U[col + PL * k];
+    if (a.sub) {
+      const int xy = (int)((i == 0 && ex > 0) || (i == N - 1 && ex < a.nx - 1)) +
+                     (int)((j == 0 && ey > 0) || (j == N - 1 && ey < a.ny - 1));
+#pragma unroll
+      for (int k = 0; k < N; ++k) {
+        const int zi = (int)((k == 0 && ez > 0) || (k == N - 1 && ez < a.nz - 1));
+        const double w = __longlong_as_double((long long)(1023 - xy - zi) << 52);
+        yv[k] = valid ? a.sub[eb + N2 * k] * w - yv[k] : 0.0;
+      }
+    }
+    // x-interfaces inside the block: (N - 1, j, k) of element lp and (0, j, k) of lp + 1 when both
+    // lie in one row; both copies get left + right.  Each pair is added once, by one lane of
+    // densely packed warps (a warp-wide FP64 instruction costs the same with 2 or 32 lanes active)
+    const bool left = i == N - 1 && le + 1 < a.NE && e + 1 < a.E && ex < a.nx - 1;
+    const bool right = i == 0 && le > 0 && ex > 0;
+    if (left || right) {
+#pragma unroll
+      for (int k = 0; k < N; ++k) U[col + PL * k] = yv[k];
+    }
+    __syncthreads();
+    const int64_t e0 = (int64_t)blockIdx.x * a.NE;
+    for (int idx = threadIdx.x; idx < (a.NE - 1) * N2; idx += blockDim.x) {
+      const int lp = idx / N2, jk = idx - lp * N2;
+      const int el = (int)(e0 + lp);
+      if (el + 1 < a.E && el % a.nx < a.nx - 1) {
+        double* p = reinterpret_cast<double*>(smem_raw) + (size_t)lp * 3 * VOL + NP * jk + N - 1;
+        double* q = p + 3 * VOL - (N - 1);
+        const double v = *p + *q;
+        *p = v;
+        *q = v;
+      }
+    }
+    __syncthreads();
+    if (left || right) {
+#pragma unroll
+      for (int k = 0; k < N; ++k) yv[k] = U[col + PL * k];
+    }
+    if (valid) {
+#pragma unroll
+      for (int k = 0; k < N; ++k) a.y[eb + N2 * k] = ((zmask >> k) & 1u) ? 0.0 : yv[k];
+    }
+  } else {
+    if (valid) {
+#pragma unroll
+      for (int k = 0; k < N; ++k) a.y[eb + N2 * k] = ax_output(U[col + PL * k], a.sub, a.pflag, eb + N2 * k);
+    }
+  }
+}
+
+// The x-interfaces that ax_fx_kernel<FOLD> leaves: element e = (b + 1) NE - 1, the last of block b,
+// and e + 1, the first of block b + 1, when both lie in one row.  Thread: (boundary, point (j, k)
+// of the face).  Masked copies are zero on both sides (a node's copies are all masked or none).
+template <int N>
+__global__ void gs_fold_fixup_x(int64_t E, int NE, int nx, double* __restrict__ y) {
+  constexpr int N2 = N * N, N3 = N2 * N;
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t nbnd = (E + NE - 1) / NE - 1;
+  if (t >= nbnd * N2) return;
+  const int64_t b = t / N2;
+  const int jk = (int)(t - b * N2);
+  const int64_t e = (b + 1) * NE - 1;
+  if (e + 1 >= E || (int)(e % nx) == nx - 1) return;
+  const int64_t ia = e * N3 + (N - 1) + (int64_t)N * jk;  // (N - 1, j, k) of e
+  const int64_t ib = (e + 1) * N3 + (int64_t)N * jk;      // (0, j, k) of e + 1
+  const double v = y[ia] + y[ib];
+  y[ia] = v;
+  y[ib] = v;
+}
+
+template <int N>
+static int launch_ax_fx(const Level& lv, const double* u, double* y, bool mask_in, const double* sub,
+                        const double* dinv, int NE, bool fold, cudaStream_t s) {
+  static_assert(sizeof(FxFold<N, N>) <= 1536, "two folded tables and the arguments fit the 4 KB of parameters");
+  double Dt[N * N];
+  for (int r = 0; r < N; ++r)
+    for (int c = 0; c < N; ++c) Dt[r * N + c] = lv.basis.D[c * N + r];
+  const FxFold<N, N> tD = fx_fold_tables<N, N>(lv.basis.D), tT = fx_fold_tables<N, N>(Dt);
+  AxFxArgs a{};
+  a.E = lv.E;
+  a.L = lv.L;
+  a.NE = NE;
+  a.u = u;
+  a.G = lv.G64;
+  a.D = lv.D64;
+  a.sub = sub;
+  a.dinv = dinv;
+  a.pflag = lv.pflag;
+  a.y = y;
+  a.mask_in = mask_in;
+  const int threads = NE * N * N;
+  const size_t smem = (size_t)NE * (3 * AxFxDims<N>::VOL * sizeof(double) + 2 * sizeof(unsigned));
+  const unsigned blocks = (unsigned)((lv.E + NE - 1) / NE);
+  if (fold) {
+    a.nx = lv.nel[0];
+    a.ny = lv.nel[1];
+    a.nz = lv.nel[2];
+    for (int f = 0; f < 6; ++f)
+      if (lv.bc[f] == SE_BC_DIRICHLET) a.bits |= 1 << f;
+    static const cudaError_t attr = cudaFuncSetAttribute(
+        ax_fx_kernel<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    SE_CUDA(attr);
+    ax_fx_kernel<N, true><<<blocks, threads, smem, s>>>(a, tD, tT);
+  } else {
+    static const cudaError_t attr = cudaFuncSetAttribute(
+        ax_fx_kernel<N, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    SE_CUDA(attr);
+    ax_fx_kernel<N, false><<<blocks, threads, smem, s>>>(a, tD, tT);
+  }
+  SE_LAUNCH_CHECK();
+  return SE_OK;
+}
+
+// y = A_L (dinv .* u), or sub / multiplicity minus it.  fold: with the x-interface sums of the
+// block's elements and the mask of the box lattice (NE elements per block).
+int ax_local_fx(const Level& lv, const double* u, double* y, bool mask_in, const double* sub,
+                const double* dinv, int NE, bool fold, cudaStream_t s) {
+  switch (lv.N) {
+#define SE_AXFX_CASE(NN) \
+  case NN: return launch_ax_fx<NN>(lv, u, y, mask_in, sub, dinv, NE, fold, s);
+    SE_AXFX_CASE(2) SE_AXFX_CASE(3) SE_AXFX_CASE(4) SE_AXFX_CASE(5) SE_AXFX_CASE(6)
+    SE_AXFX_CASE(7) SE_AXFX_CASE(8) SE_AXFX_CASE(9) SE_AXFX_CASE(10) SE_AXFX_CASE(11)
+#undef SE_AXFX_CASE
+    default: set_error("ax: unsupported N=%d", lv.N); return SE_EINVAL;
+  }
+}
+
+int gs_fold_fixup(const Level& lv, double* y, int NE, cudaStream_t s) {
+  const int64_t nbnd = (lv.E + NE - 1) / NE - 1;
+  if (nbnd <= 0 || lv.nel[0] <= 1) return SE_OK;
+  const int64_t n = nbnd * lv.N * lv.N;
+  switch (lv.N) {
+#define SE_FIX_CASE(NN)                                                                      \
+  case NN:                                                                                   \
+    gs_fold_fixup_x<NN><<<grid_for(n, 256), 256, 0, s>>>(lv.E, NE, lv.nel[0], y);            \
+    break;
+    SE_FIX_CASE(2) SE_FIX_CASE(3) SE_FIX_CASE(4) SE_FIX_CASE(5) SE_FIX_CASE(6)
+    SE_FIX_CASE(7) SE_FIX_CASE(8) SE_FIX_CASE(9) SE_FIX_CASE(10) SE_FIX_CASE(11)
+#undef SE_FIX_CASE
+    default: set_error("gs_fold_fixup: unsupported N=%d", lv.N); return SE_EINVAL;
+  }
+  SE_LAUNCH_CHECK();
+  return SE_OK;
+}
+
+}  // namespace se

@@ -1,0 +1,286 @@
+// FP64-accurate line contractions on the integer pipe (block floating point).
+//
+// GB300 executes 2 FP64 FMAs per clock and SM, but about 36 32 x 32 + 64 bit integer multiply-adds
+// (IMAD.WIDE, measured with independent chains: 36 lanes/clk/SM against 1.6-2 of DFMA).  A
+// contraction out_i = sum_l M_il v_l whose inputs share one binary scale is therefore cheaper in
+// fixed point: three integer multiply-adds per term instead of one DFMA, 7 times the rate.
+//
+//   value      x = v 2^(56 - e), |x| < 2^57, e the (unbiased) exponent of the largest |v| of the
+//              element: kept as x = h 2^28 + l, h signed, 0 <= l <= 2^28 (fx_split; bits below
+//              2^-56 of the largest value are dropped)
+//   matrix     M' = M 2^k rounded to an integer, |M'| < 2^59 and sum_l |M'_il| < 2^60, kept as
+//              mh 2^28 + ml with -2^27 <= ml < 2^27 (fx_limbs)
+//   product    hi = sum mh h, mid = sum (mh l + ml h), 64-bit sums that cannot overflow
+//              (|hi| < 2^61, |mid| < 2^62); the ml l terms (below 2^-59 of the largest
+//              possible sum) are left out.  R = hi + floor(mid / 2^28), |R| < 2^61, is the
+//              result in units of 2^(e - k) (three such sums may be added in 64 bits)
+//   back       the double nearest to R 2^(e - k) (fx_double): one rounding to 53 bits
+//
+// Every error is below 2^-56 of (largest value of the element) x (largest row sum of M); an FP64
+// dot product rounds each of its terms to 2^-53 of the running sum.  Exponents outside
+// [FX_EMIN, FX_EMAX] (infinities, NaN, values whose results could leave the normal range) are not
+// representable: kernels test for them and compute such elements in FP64.
+//
+// The arithmetic also compiles as host code, so that its accuracy can be checked without a GPU.
+#pragma once
+#include <cstdint>
+#include <cstring>
+
+#ifdef __CUDACC__
+#define SE_FX __host__ __device__ __forceinline__
+#else
+#define SE_FX inline
+#endif
+
+namespace se {
+
+constexpr int FX_LIMB = 28;
+constexpr int FX_EMIN = 70, FX_EMAX = 2020;  // biased exponents of the largest value
+
+// Folded tables of a centro-(anti)symmetric N x N matrix M, M[N-1-k][N-1-l] = sym * M[k][l]:
+// with e_l = v_l + v_{N-1-l}, o_l = v_l - v_{N-1-l} (l < N/2; for odd N also e_m = v_m, m = N/2)
+//   2 (M v)_k       =  E_k + O_k         E_k = sum_l (M_kl + M_k,N-1-l) e_l   (middle: 2 M_km e_m)
+//   2 (M v)_{N-1-k} = sym (E_k - O_k)    O_k = sum_l (M_kl - M_k,N-1-l) o_l
+// The tables hold 2^k (M_kl +- M_k,N-1-l) as limbs; `k` includes the factor 2.  A kernel takes
+// them as a parameter, so that every multiplier is a constant-bank operand.
+template <int NR, int NC>
+struct FxFold {
+  static constexpr int RE = (NR + 1) / 2;  // rows computed (the others follow by symmetry)
+  static constexpr int CE = (NC + 1) / 2, CO = NC / 2;
+  int eh[RE * CE], el[RE * CE];
+  int oh[RE * (CO > 0 ? CO : 1)], ol[RE * (CO > 0 ? CO : 1)];
+  int k;
+};
+
+// ------------------------------------------------------------------ word operations
+SE_FX void fx_words(double v, unsigned& hi, unsigned& lo) {
+#ifdef __CUDA_ARCH__
+  hi = (unsigned)__double2hiint(v);
+  lo = (unsigned)__double2loint(v);
+#else
+  unsigned long long b;
+  std::memcpy(&b, &v, 8);
+  hi = (unsigned)(b >> 32);
+  lo = (unsigned)b;
+#endif
+}
+SE_FX double fx_from_words(unsigned hi, unsigned lo) {
+#ifdef __CUDA_ARCH__
+  return __hiloint2double((int)hi, (int)lo);
+#else
+  const unsigned long long b = ((unsigned long long)hi << 32) | lo;
+  double v;
+  std::memcpy(&v, &b, 8);
+  return v;
+#endif
+}
+// High word of (hi, lo) << n and low word of (hi, lo) >> n, n modulo 32.
+SE_FX unsigned fx_funnel_l(unsigned lo, unsigned hi, int n) {
+#ifdef __CUDA_ARCH__
+  return __funnelshift_l(lo, hi, n);
+#else
+  return (unsigned)(((((unsigned long long)hi << 32) | lo) << (n & 31)) >> 32);
+#endif
+}
+SE_FX unsigned fx_funnel_r(unsigned lo, unsigned hi, int n) {
+#ifdef __CUDA_ARCH__
+  return __funnelshift_r(lo, hi, n);
+#else
+  return (unsigned)((((unsigned long long)hi << 32) | lo) >> (n & 31));
+#endif
+}
+// x >> n; 0 (or the sign) for n >= 64.
+SE_FX unsigned long long fx_shr(unsigned long long x, int n) {
+#ifdef __CUDA_ARCH__
+  asm("shr.u64 %0, %0, %1;" : "+l"(x) : "r"(n));
+  return x;
+#else
+  return n > 63 ? 0ull : x >> n;
+#endif
+}
+SE_FX long long fx_shr(long long x, int n) {
+#ifdef __CUDA_ARCH__
+  asm("shr.s64 %0, %0, %1;" : "+l"(x) : "r"(n));
+  return x;
+#else
+  return x >> (n > 63 ? 63 : n);
+#endif
+}
+// Position of the leading bit, -1 for 0.
+SE_FX int fx_bfind(unsigned x) {
+#ifdef __CUDA_ARCH__
+  int p;
+  asm("bfind.u32 %0, %1;" : "=r"(p) : "r"(x));
+  return p;
+#else
+  return x ? 31 - __builtin_clz(x) : -1;
+#endif
+}
+
+// ------------------------------------------------------------------ tables
+// Limbs of an integer |m| < 2^59 - 2^27.
+SE_FX void fx_limbs(long long m, int& mh, int& ml) {
+  const long long h = (m + (1ll << (FX_LIMB - 1))) >> FX_LIMB;
+  mh = (int)h;
+  ml = (int)(m - (h << FX_LIMB));
+}
+
+// Folded fixed-point tables of M (row-major NR x NC), host.
+template <int NR, int NC>
+inline FxFold<NR, NC> fx_fold_tables(const double* M) {
+  FxFold<NR, NC> t{};
+  double rows = 0.0;
+  for (int r = 0; r < NR; ++r) {
+    double s = 0.0;
+    for (int c = 0; c < NC; ++c) s += M[r * NC + c] < 0 ? -M[r * NC + c] : M[r * NC + c];
+    rows = s > rows ? s : rows;
+  }
+  // rows 2^k < 2^58: then a folded entry is below 2^58 and a folded row sum below 2^59
+  int k = 0;
+  while (rows >= 288230376151711744.0) rows *= 0.5, --k;
+  while (rows * 2.0 < 288230376151711744.0) rows *= 2.0, ++k;
+  double scale = 1.0;
+  for (int q = 0; q < k; ++q) scale *= 2.0;
+  for (int q = 0; q > k; --q) scale *= 0.5;
+  auto fix = [&](int r, int c) {
+    const double m = M[r * NC + c] * scale;
+    return (long long)(m < 0 ? m - 0.5 : m + 0.5);
+  };
+  for (int r = 0; r < t.RE; ++r) {
+    for (int c = 0; c < t.CE; ++c) fx_limbs(fix(r, c) + fix(r, NC - 1 - c), t.eh[r * t.CE + c], t.el[r * t.CE + c]);
+    for (int c = 0; c < t.CO; ++c) fx_limbs(fix(r, c) - fix(r, NC - 1 - c), t.oh[r * t.CO + c], t.ol[r * t.CO + c]);
+  }
+  t.k = k + 1;
+  return t;
+}
+
+// ------------------------------------------------------------------ values
+// High word without the sign: orders doubles by magnitude.
+SE_FX unsigned fx_mag(double v) {
+  unsigned hi, lo;
+  fx_words(v, hi, lo);
+  return hi & 0x7fffffffu;
+}
+
+// Biased exponent of an element whose largest fx_mag is `mag`, and whether it can be represented
+// (an element of zeros is; one whose largest value is below 2^-1022 x 2^-20 counts as zeros).
+SE_FX int fx_exponent(unsigned mag) {
+  const int e = (int)(mag >> 20);
+  return e > FX_EMIN ? e : FX_EMIN;
+}
+SE_FX bool fx_bad(unsigned mag) {
+  return mag != 0u && (unsigned)((int)(mag >> 20) - FX_EMIN) > (unsigned)(FX_EMAX - FX_EMIN);
+}
+
+// v in units of 2^(E - 1023 - 56), E >= every value's biased exponent.
+SE_FX void fx_split(double v, int E, int& h, int& l) {
+  unsigned hi, lo;
+  fx_words(v, hi, lo);
+  const int s = (int)hi >> 31;
+  const int sh = E - (int)((hi >> 20) & 0x7ffu);
+  // 61-bit magnitude, the implicit one at bit 60 (a zero or subnormal is shifted out: sh >= 70)
+  const unsigned top = (fx_funnel_l(lo, hi, 8) & 0x0fffffffu) | 0x10000000u;
+  const unsigned long long x = fx_shr(((unsigned long long)top << 32) | (lo << 8), sh);
+  const unsigned xl = (unsigned)x >> 4;
+  h = (int)(unsigned)(x >> 32) ^ s;
+  l = (int)((xl ^ (unsigned)s) & 0x0fffffffu) - s;
+}
+
+// The double nearest to R 2^(eb - 1023), |R| < 2^62; eb >= 1 and eb + 63 < 2046 (callers bound
+// the exponents).  Normalisation by the position of the leading bit, rounding by adding half a
+// unit before the cut (a carry moves into the exponent field).  Up to two units of R are dropped:
+// one where R < 0 (|R| as the one's complement), one where |R| < 2^32.  No branches: the
+// conversions of a line's results interleave.
+SE_FX double fx_double(long long R, int eb) {
+  const unsigned s = (unsigned)((int)(R >> 32) >> 31);
+  const unsigned rh = (unsigned)((unsigned long long)R >> 32) ^ s, rl = (unsigned)R ^ s;
+  const bool small = rh == 0u;
+  unsigned h = small ? rl >> 1 : rh, l = small ? 0u : rl;
+  const int p = small ? eb : eb + 31;
+  const int pos = fx_bfind(h);
+  const int n = 30 - pos;
+  const unsigned mh0 = fx_funnel_l(l, h, n);
+  l <<= n & 31;  // leading bit at bit 62 of (mh0, l)
+  const unsigned long long m = (((unsigned long long)mh0 << 32) | l) + 0x200u;
+  const unsigned mh = (unsigned)(m >> 32);
+  const unsigned lo = fx_funnel_r((unsigned)m, mh, 10);
+  const unsigned hi = (mh >> 10) + ((unsigned)(p + pos) << 20);
+  return fx_from_words(h ? hi | (s & 0x80000000u) : 0u, h ? lo : 0u);
+}
+
+// ------------------------------------------------------------------ renormalisation of 64-bit results
+// |R| by its high word (one less for negative R).
+SE_FX unsigned fx_high(long long R) {
+  const int h = (int)(R >> 32);
+  return (unsigned)(h ^ (h >> 31));
+}
+
+// Left shift that brings values whose largest high word is `high` to 63 bits.
+SE_FX int fx_norm(unsigned high) { return high ? 30 - fx_bfind(high) : 30; }
+
+// Limbs of R after a left shift by n, in units 2^6: x = R 2^n / 2^6, |x| < 2^57.
+SE_FX void fx_renorm(long long R, int n, int& h, int& l) {
+  const unsigned long long x = (unsigned long long)R << n;
+  const int xh = (int)(x >> 32);
+  h = xh >> 2;
+  l = (int)(fx_funnel_r((unsigned)x, (unsigned)xh, 6) & 0x0fffffffu);
+}
+
+#ifdef __CUDACC__
+// Starts moving n doubles at p towards L2 (whole 16-byte units inside [p - 1, p + n)).
+__device__ __forceinline__ void fx_prefetch(const double* p, int n) {
+  const unsigned long long a = (unsigned long long)p & ~15ull;
+  const unsigned bytes = (unsigned)(((unsigned long long)(p + n) - a) & ~15ull);
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"(bytes) : "memory");
+}
+#endif
+
+// R of the folded contraction of the line (h, l): out(k, R) for k < NR.  SYM = -1: M is
+// centro-antisymmetric (derivatives), +1: centro-symmetric (interpolation).
+template <int NR, int NC, int SYM, class Out>
+SE_FX void fx_contract(const FxFold<NR, NC>& t, const int (&h)[NC], const int (&l)[NC],
+                                            Out&& out) {
+  constexpr int RE = FxFold<NR, NC>::RE, CE = FxFold<NR, NC>::CE, CO = FxFold<NR, NC>::CO;
+  int eh[CE], el[CE], oh[CE], ol[CE];
+#pragma unroll
+  for (int c = 0; c < CO; ++c) {
+    eh[c] = h[c] + h[NC - 1 - c];
+    el[c] = l[c] + l[NC - 1 - c];
+    oh[c] = h[c] - h[NC - 1 - c];
+    ol[c] = l[c] - l[NC - 1 - c];
+  }
+  if constexpr (CE > CO) {
+    eh[CO] = h[CO];
+    el[CO] = l[CO];
+  }
+#pragma unroll
+  for (int r = 0; r < RE; ++r) {
+    const bool mid = NR % 2 == 1 && r == RE - 1;  // the middle row is its own mirror image
+    long long hE = 0, mE = 0, hO = 0, mO = 0;
+    if (!(mid && SYM < 0)) {
+#pragma unroll
+      for (int c = 0; c < CE; ++c) {
+        hE += (long long)t.eh[r * CE + c] * eh[c];
+        mE += (long long)t.eh[r * CE + c] * el[c];
+        mE += (long long)t.el[r * CE + c] * eh[c];
+      }
+    }
+    if (!(mid && SYM > 0)) {
+#pragma unroll
+      for (int c = 0; c < CO; ++c) {
+        hO += (long long)t.oh[r * CO + c] * oh[c];
+        mO += (long long)t.oh[r * CO + c] * ol[c];
+        mO += (long long)t.ol[r * CO + c] * oh[c];
+      }
+    }
+    if (mid) {
+      out(r, SYM < 0 ? hO + (mO >> FX_LIMB) : hE + (mE >> FX_LIMB));
+    } else {
+      const long long E = hE + (mE >> FX_LIMB), O = hO + (mO >> FX_LIMB);
+      out(r, E + O);
+      out(NR - 1 - r, SYM < 0 ? O - E : E - O);
+    }
+  }
+}
+
+}  // namespace se

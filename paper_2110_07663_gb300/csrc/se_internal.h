@@ -234,8 +234,9 @@ int build_level_gsmap(Level& lv, Allocs& allocs, cudaStream_t s);
 // blocks, then the y/z launch follow (ax.cu).
 bool ax_fold_ok(const Level& lv);
 // dinv: y = A (dinv .* u) (the input scaled as it is loaded)
+// mask_in: u may be non-zero on Dirichlet nodes (zeroed as it is loaded)
 int ax_apply_folded(const Level& lv, const double* u, double* y, const double* b, cudaStream_t s,
-                    const double* dinv = nullptr);
+                    const double* dinv = nullptr, bool mask_in = false);
 template <class T>
 inline int ax_apply(const Level& lv, const T* u, T* y, cudaStream_t s) {
   if constexpr (sizeof(T) == 8)
@@ -388,14 +389,15 @@ int ax_elems_per_block(int p, bool fp32);
 bool ax_tma_supported(int p);
 int ax_tma_group(int p);
 int ax_local_tma(const Level& lv, const float* u, float* y, cudaStream_t s, const float* sub);
-// FP64 Ax with even-odd folded contractions (even N).
+// FP64 Ax (block floating point, ax_fx.cu): y = A_L (dinv .* u), or sub / multiplicity minus it;
+// dinv and sub may be null.  fold: with the x-interface sums of the block's elements (NE per
+// block) and the mask.
+int ax_local_fx(const Level& lv, const double* u, double* y, bool mask_in, const double* sub,
+                const double* dinv, int NE, bool fold, cudaStream_t s);
+// Even-odd folded df64 kernel (even N).
 bool ax_eo_supported(int p);
 void ax_eo_tables(const Basis1D& b, double* out);
-int ax_local_eo(const Level& lv, const double* u, double* y, cudaStream_t s, const double* sub);
-// The same with the x-interface sums of the block's elements and the mask (NE elements per block).
-int ax_local_eo_fold(const Level& lv, const double* u, double* y, const double* sub, int NE,
-                     cudaStream_t s, const double* dinv = nullptr);
-// The x-interfaces between consecutive blocks of ax_local_eo_fold (NE elements per block).
+// The x-interfaces between consecutive blocks of ax_local_fx with fold (NE elements per block).
 int gs_fold_fixup(const Level& lv, double* y, int NE, cudaStream_t s);
 // The same contractions in df64 arithmetic (FP64 in and out); needs lv.Gdf and lv.eodf.
 int ax_local_eo_df(const Level& lv, const double* u, double* y, cudaStream_t s, const double* sub);
