@@ -1,11 +1,12 @@
 // FP64 local Ax with folded line contractions in block floating point (fxp.h), every N.
 //
 // Sum factorisation: (ur, us, ut) = (D_r u, D_s u, D_t u);  w = G (ur, us, ut);
-// y = D_r^T wr + D_s^T ws + D_t^T wt.  The six contractions run on the integer pipe: u is split
-// once into fixed point on the scale of the element's largest value, the gradients come back as
-// doubles for the pointwise product with G (9 FP64 instructions per point, what is left on the
-// FP64 pipe), w is split again on its own scale, and the three parts of y are added as 64-bit
-// integers before the one rounding to double.  The derivative matrix is centro-antisymmetric, so
+// y = D_r^T wr + D_s^T ws + D_t^T wt.  The six contractions run on the integer pipe: a line of u is
+// split into fixed point on the scale of its largest value (so that a result's error is relative to
+// its own line, as in FP64), the gradients come back as doubles for the pointwise product with G
+// (9 FP64 instructions per point, what is left on the FP64 pipe), w is split on the scale of the
+// element's largest value, and the three parts of y are added as 64-bit integers before the one
+// rounding to double.  The derivative matrix is centro-antisymmetric, so
 // a line of N values costs N^2/2 terms.
 //
 // NE elements per block, N^2 threads per element; each thread owns one line per direction.  Per
@@ -21,11 +22,16 @@
 // left to gs_fold_fixup_x.
 //
 // Measured on GB300 (us per launch; in brackets the even-odd FP64 kernel this one replaced, which ran at
-// the FP64 pipe's 2 FMA/clk/SM): 32^3 elements p = 7 417 [1420], p = 5 187 [525], p = 3 56 [138]; even
-// orders (unfolded in FP64) 20^3 p = 8 202 [725].  Memory needs 158 us of the 417, the 9 FP64
+// the FP64 pipe's 2 FMA/clk/SM): 32^3 elements p = 7 429 [1420], p = 5 196 [525], p = 3 57 [138]; even
+// orders (unfolded in FP64) 20^3 p = 8 192 [725].  Memory needs 158 us of the 429, the 9 FP64
 // instructions per point 240, and the integer pipes about the same: what is left are the waits between
-// them, so resident warps count (64 registers: 417, 80: 440, 128: 485; before the conversions back
-// were branch-free and G was prefetched to L2, 530 to 560).
+// them, so resident warps count (64 registers: 429, 80: 456, 96: 482; before the conversions back
+// were branch-free and G was prefetched to L2, 530 to 560).  u on the element's scale instead of each
+// line's was 4% faster, but lost accuracy where values within an element span many decades.
+//
+// Error against extended precision (2-norm, on this repository's meshes), over that of the FP64 dot
+// products: 0.6 to 0.75 for random values, 0.3 to 0.8 for smooth ones, 0.6 for values that decay by
+// eight decades across the element.
 //
 // Elements whose values cannot share a scale (infinities, NaN, magnitudes at the ends of the
 // range) send their block to ax_slow_block, the same operator in FP64.
@@ -43,6 +49,23 @@ struct AxFxArgs {
   int mask_in;             // zero the Dirichlet values of u as they are read
   int nx, ny, nz, bits;    // FOLD
 };
+
+// Splits the line p[0], p[st], ... on its own scale and calls f(E); whether it could not.
+template <int N, class F>
+__device__ __forceinline__ bool fx_split_line(const double* p, int st, int (&h)[N], int (&l)[N], F&& f) {
+  double v[N];
+  unsigned mag = 0u;
+#pragma unroll
+  for (int q = 0; q < N; ++q) {
+    v[q] = p[st * q];
+    mag = max(mag, fx_mag(v[q]));
+  }
+  const int E = fx_exponent(mag);
+#pragma unroll
+  for (int q = 0; q < N; ++q) fx_split(v[q], E, h[q], l[q]);
+  f(E);
+  return fx_bad(mag);
+}
 
 template <int N>
 struct AxFxDims {
@@ -130,7 +153,7 @@ __global__ void __maxnreg__(ax_fx_regs<N>())
   const bool valid = e < a.E;
   const int64_t eb = e * N3 + t;
   const int col = i + NP * j, rl = NP * i + PL * j, sl = i + PL * j;  // lines: column, (j=i,k=j), (i,k=j)
-  if (t == 0) mags[2 * le] = mags[2 * le + 1] = 0u;
+  if (t == 0) mags[le] = 0u;
   // the geometric factors are needed after the forward contractions: on their way to L2 meanwhile
   if (valid && t < 6 && N2 >= 6) fx_prefetch(a.G + t * a.L + e * N3, N3);
   // Dirichlet points of the column (bit k)
@@ -152,58 +175,38 @@ __global__ void __maxnreg__(ax_fx_regs<N>())
       if (!(a.pflag[eb + N2 * k] & PF_FREE)) zmask |= 1u << k;
   }
   const unsigned zin = a.mask_in ? zmask : 0u;
-  __syncthreads();
   bool bad = false;
+  int Et;  // scale of the thread's column
   {
-    double v[N];
     unsigned mag = 0u;
 #pragma unroll
     for (int k = 0; k < N; ++k) {
-      v[k] = valid ? ax_fx_input(a, eb + N2 * k, (zin >> k) & 1u) : 0.0;
-      mag = max(mag, fx_mag(v[k]));
+      const double v = valid ? ax_fx_input(a, eb + N2 * k, (zin >> k) & 1u) : 0.0;
+      U[col + PL * k] = v;
+      mag = max(mag, fx_mag(v));
     }
-    if (mag) atomicMax(&mags[2 * le], mag);
-    __syncthreads();
-    mag = mags[2 * le];
     bad = fx_bad(mag);
-    const int E = fx_exponent(mag);
-#pragma unroll
-    for (int k = 0; k < N; ++k) {
-      int h, l;
-      fx_split(v[k], E, h, l);
-      reinterpret_cast<int2*>(U)[col + PL * k] = make_int2(h, l);
-    }
+    Et = fx_exponent(mag);
+  }
+  __syncthreads();
+  // r-lines and s-lines
+  {
+    int h[N], l[N];
+    bad |= fx_split_line<N>(U + rl, 1, h, l, [&](int E) {
+      fx_contract<N, N, -1>(tD, h, l, [&](int q, long long r) { R[rl + q] = fx_double(r, E - tD.k); });
+    });
+    bad |= fx_split_line<N>(U + sl, NP, h, l, [&](int E) {
+      fx_contract<N, N, -1>(tD, h, l, [&](int q, long long r) { S[sl + NP * q] = fx_double(r, E - tD.k); });
+    });
   }
   bad = __syncthreads_or(bad);
   if (!bad) {
-    const int eb1 = fx_exponent(mags[2 * le]) - tD.k;
-    {
-      int h[N], l[N];
-#pragma unroll
-      for (int q = 0; q < N; ++q) {
-        const int2 x = reinterpret_cast<const int2*>(U)[rl + q];
-        h[q] = x.x;
-        l[q] = x.y;
-      }
-      fx_contract<N, N, -1>(tD, h, l, [&](int q, long long r) { R[rl + q] = fx_double(r, eb1); });
-#pragma unroll
-      for (int q = 0; q < N; ++q) {
-        const int2 x = reinterpret_cast<const int2*>(U)[sl + NP * q];
-        h[q] = x.x;
-        l[q] = x.y;
-      }
-      fx_contract<N, N, -1>(tD, h, l, [&](int q, long long r) { S[sl + NP * q] = fx_double(r, eb1); });
-    }
-    __syncthreads();
     // t-lines and the pointwise factors: the thread's column
     {
+      const int eb1 = Et - tD.k;
       int h[N], l[N];
 #pragma unroll
-      for (int q = 0; q < N; ++q) {
-        const int2 x = reinterpret_cast<const int2*>(U)[col + PL * q];
-        h[q] = x.x;
-        l[q] = x.y;
-      }
+      for (int q = 0; q < N; ++q) fx_split(U[col + PL * q], Et, h[q], l[q]);
       unsigned mag = 0u;
       fx_contract<N, N, -1>(tD, h, l, [&](int q, long long r) {
         const double ut = fx_double(r, eb1), ur = R[col + PL * q], us = S[col + PL * q];
@@ -220,10 +223,10 @@ __global__ void __maxnreg__(ax_fx_regs<N>())
         U[col + PL * q] = wt;
         mag = max(max(mag, fx_mag(wr)), max(fx_mag(ws), fx_mag(wt)));
       });
-      if (mag) atomicMax(&mags[2 * le + 1], mag);
+      if (mag) atomicMax(&mags[le], mag);
     }
     __syncthreads();
-    const unsigned mag2 = mags[2 * le + 1];
+    const unsigned mag2 = mags[le];
     const int E2 = fx_exponent(mag2);
     {
       int h[N], l[N];
@@ -331,7 +334,8 @@ static int launch_ax_fx(const Level& lv, const double* u, double* y, bool mask_i
   double Dt[N * N];
   for (int r = 0; r < N; ++r)
     for (int c = 0; c < N; ++c) Dt[r * N + c] = lv.basis.D[c * N + r];
-  const FxFold<N, N> tD = fx_fold_tables<N, N>(lv.basis.D), tT = fx_fold_tables<N, N>(Dt);
+  // three results of D^T are added in 64 bits
+  const FxFold<N, N> tD = fx_fold_tables<N, N>(lv.basis.D, -1, 60), tT = fx_fold_tables<N, N>(Dt, -1, 59);
   AxFxArgs a{};
   a.E = lv.E;
   a.L = lv.L;
@@ -345,7 +349,7 @@ static int launch_ax_fx(const Level& lv, const double* u, double* y, bool mask_i
   a.y = y;
   a.mask_in = mask_in;
   const int threads = NE * N * N;
-  const size_t smem = (size_t)NE * (3 * AxFxDims<N>::VOL * sizeof(double) + 2 * sizeof(unsigned));
+  const size_t smem = (size_t)NE * (3 * AxFxDims<N>::VOL * sizeof(double) + sizeof(unsigned));
   const unsigned blocks = (unsigned)((lv.E + NE - 1) / NE);
   if (fold) {
     a.nx = lv.nel[0];

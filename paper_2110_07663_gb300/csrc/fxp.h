@@ -6,18 +6,18 @@
 // fixed point: three integer multiply-adds per term instead of one DFMA, 7 times the rate.
 //
 //   value      x = v 2^(56 - e), |x| < 2^57, e the (unbiased) exponent of the largest |v| of the
-//              element: kept as x = h 2^28 + l, h signed, 0 <= l <= 2^28 (fx_split; bits below
+//              line or element: kept as x = h 2^28 + l, h signed, 0 <= l <= 2^28 (fx_split; bits below
 //              2^-56 of the largest value are dropped)
-//   matrix     M' = M 2^k rounded to an integer, |M'| < 2^59 and sum_l |M'_il| < 2^60, kept as
-//              mh 2^28 + ml with -2^27 <= ml < 2^27 (fx_limbs)
+//   matrix     M' = M 2^k rounded to an integer, |M'| < 2^59, kept as mh 2^28 + ml with
+//              -2^27 <= ml < 2^27 (fx_limbs), its row sums bounded so that the sums below fit
 //   product    hi = sum mh h, mid = sum (mh l + ml h), 64-bit sums that cannot overflow
-//              (|hi| < 2^61, |mid| < 2^62); the ml l terms (below 2^-59 of the largest
-//              possible sum) are left out.  R = hi + floor(mid / 2^28), |R| < 2^61, is the
-//              result in units of 2^(e - k) (three such sums may be added in 64 bits)
+//              (|hi|, |mid| < 2^63); the ml l terms (below 2^-59 of the largest
+//              possible sum, and without a bias because ml has both signs) are left out.
+//              R = hi + round(mid / 2^28) is the result in units of 2^(e - k)
 //   back       the double nearest to R 2^(e - k) (fx_double): one rounding to 53 bits
 //
-// Every error is below 2^-56 of (largest value of the element) x (largest row sum of M); an FP64
-// dot product rounds each of its terms to 2^-53 of the running sum.  Exponents outside
+// Before the final rounding every error is below 2^-55 of (largest value on the scale) x (largest row
+// sum of M); an FP64 dot product rounds each of its terms to 2^-53 of the running sum.  Exponents outside
 // [FX_EMIN, FX_EMAX] (infinities, NaN, values whose results could leave the normal range) are not
 // representable: kernels test for them and compute such elements in FP64.
 //
@@ -35,6 +35,7 @@
 namespace se {
 
 constexpr int FX_LIMB = 28;
+constexpr long long FX_HALF = 1ll << (FX_LIMB - 1);  // where a middle sum starts: its cut rounds
 constexpr int FX_EMIN = 70, FX_EMAX = 2020;  // biased exponents of the largest value
 
 // Folded tables of a centro-(anti)symmetric N x N matrix M, M[N-1-k][N-1-l] = sym * M[k][l]:
@@ -125,26 +126,33 @@ SE_FX void fx_limbs(long long m, int& mh, int& ml) {
   ml = (int)(m - (h << FX_LIMB));
 }
 
-// Folded fixed-point tables of M (row-major NR x NC), host.
+// Folded fixed-point tables of M (row-major NR x NC, M[NR-1-r][NC-1-c] = sym M[r][c] up to rounding:
+// both entries are averaged), host.  rows_log2: the largest row sum of |M'| stays below 2^rows_log2,
+// at most 60; entries stay below 2^59.  |R| < 2^(rows_log2 + 2) for |x| < 2^57.
 template <int NR, int NC>
-inline FxFold<NR, NC> fx_fold_tables(const double* M) {
+inline FxFold<NR, NC> fx_fold_tables(const double* M, int sym, int rows_log2) {
   FxFold<NR, NC> t{};
-  double rows = 0.0;
+  double rows = 0.0, most = 0.0;
   for (int r = 0; r < NR; ++r) {
     double s = 0.0;
-    for (int c = 0; c < NC; ++c) s += M[r * NC + c] < 0 ? -M[r * NC + c] : M[r * NC + c];
+    for (int c = 0; c < NC; ++c) {
+      const double m = M[r * NC + c] < 0 ? -M[r * NC + c] : M[r * NC + c];
+      s += m;
+      most = m > most ? m : most;
+    }
     rows = s > rows ? s : rows;
   }
-  // rows 2^k < 2^58: then a folded entry is below 2^58 and a folded row sum below 2^59
+  // a folded entry is at most twice an entry of M, and the tables hold twice the average
+  double lim = 1.0;
+  for (int q = 0; q < rows_log2; ++q) lim *= 2.0;
   int k = 0;
-  while (rows >= 288230376151711744.0) rows *= 0.5, --k;
-  while (rows * 2.0 < 288230376151711744.0) rows *= 2.0, ++k;
-  double scale = 1.0;
-  for (int q = 0; q < k; ++q) scale *= 2.0;
-  for (int q = 0; q > k; --q) scale *= 0.5;
+  double f = 1.0;
+  auto fits = [&](double g) { return rows * g < lim && 2.0 * most * g < 576460000000000000.0; };  // 2^59
+  while (!fits(f)) f *= 0.5, --k;
+  while (fits(2.0 * f)) f *= 2.0, ++k;
   auto fix = [&](int r, int c) {
-    const double m = M[r * NC + c] * scale;
-    return (long long)(m < 0 ? m - 0.5 : m + 0.5);
+    const double m = M[r * NC + c] * f * 0.5, w = sym * M[(NR - 1 - r) * NC + (NC - 1 - c)] * f * 0.5;
+    return (long long)(m < 0 ? m - 0.5 : m + 0.5) + (long long)(w < 0 ? w - 0.5 : w + 0.5);
   };
   for (int r = 0; r < t.RE; ++r) {
     for (int c = 0; c < t.CE; ++c) fx_limbs(fix(r, c) + fix(r, NC - 1 - c), t.eh[r * t.CE + c], t.el[r * t.CE + c]);
@@ -172,21 +180,25 @@ SE_FX bool fx_bad(unsigned mag) {
   return mag != 0u && (unsigned)((int)(mag >> 20) - FX_EMIN) > (unsigned)(FX_EMAX - FX_EMIN);
 }
 
-// v in units of 2^(E - 1023 - 56), E >= every value's biased exponent.
+// v in units of 2^(E - 1023 - (XB - 1)), |x| < 2^XB, E >= every value's biased exponent.  XB = 57, or
+// 58 where lines are not folded (a folded sum needs the bit).
+template <int XB = 57>
 SE_FX void fx_split(double v, int E, int& h, int& l) {
   unsigned hi, lo;
   fx_words(v, hi, lo);
   const int s = (int)hi >> 31;
   const int sh = E - (int)((hi >> 20) & 0x7ffu);
-  // 61-bit magnitude, the implicit one at bit 60 (a zero or subnormal is shifted out: sh >= 70)
-  const unsigned top = (fx_funnel_l(lo, hi, 8) & 0x0fffffffu) | 0x10000000u;
-  const unsigned long long x = fx_shr(((unsigned long long)top << 32) | (lo << 8), sh);
+  // XB + 4 bit magnitude, led by the implicit one (a zero or subnormal is shifted out: sh >= 70)
+  constexpr int UP = XB - 49;
+  const unsigned one = 1u << (20 + UP);
+  const unsigned top = (fx_funnel_l(lo, hi, UP) & (one - 1u)) | one;
+  const unsigned long long x = fx_shr(((unsigned long long)top << 32) | (lo << UP), sh);
   const unsigned xl = (unsigned)x >> 4;
   h = (int)(unsigned)(x >> 32) ^ s;
   l = (int)((xl ^ (unsigned)s) & 0x0fffffffu) - s;
 }
 
-// The double nearest to R 2^(eb - 1023), |R| < 2^62; eb >= 1 and eb + 63 < 2046 (callers bound
+// The double nearest to R 2^(eb - 1023), |R| < 2^63; eb >= 1 and eb + 63 < 2046 (callers bound
 // the exponents).  Normalisation by the position of the leading bit, rounding by adding half a
 // unit before the cut (a carry moves into the exponent field).  Up to two units of R are dropped:
 // one where R < 0 (|R| as the one's complement), one where |R| < 2^32.  No branches: the
@@ -218,12 +230,14 @@ SE_FX unsigned fx_high(long long R) {
 // Left shift that brings values whose largest high word is `high` to 63 bits.
 SE_FX int fx_norm(unsigned high) { return high ? 30 - fx_bfind(high) : 30; }
 
-// Limbs of R after a left shift by n, in units 2^6: x = R 2^n / 2^6, |x| < 2^57.
+// Limbs of R after a left shift by n to 63 bits: x = R 2^n / 2^(63 - XB), |x| < 2^XB.
+template <int XB = 57>
 SE_FX void fx_renorm(long long R, int n, int& h, int& l) {
   const unsigned long long x = (unsigned long long)R << n;
   const int xh = (int)(x >> 32);
-  h = xh >> 2;
-  l = (int)(fx_funnel_r((unsigned)x, (unsigned)xh, 6) & 0x0fffffffu);
+  constexpr int DOWN = 63 - XB;
+  h = xh >> (DOWN + FX_LIMB - 32);
+  l = (int)(fx_funnel_r((unsigned)x, (unsigned)xh, DOWN) & 0x0fffffffu);
 }
 
 #ifdef __CUDACC__
@@ -256,7 +270,7 @@ SE_FX void fx_contract(const FxFold<NR, NC>& t, const int (&h)[NC], const int (&
 #pragma unroll
   for (int r = 0; r < RE; ++r) {
     const bool mid = NR % 2 == 1 && r == RE - 1;  // the middle row is its own mirror image
-    long long hE = 0, mE = 0, hO = 0, mO = 0;
+    long long hE = 0, mE = FX_HALF, hO = 0, mO = FX_HALF;
     if (!(mid && SYM < 0)) {
 #pragma unroll
       for (int c = 0; c < CE; ++c) {

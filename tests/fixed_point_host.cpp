@@ -32,7 +32,7 @@ static void lines(int spread, int shift) {
       v[c] = std::ldexp(uniform(), shift - (int)(rng() % (spread + 1)));
       vmax = std::fmax(vmax, std::fabs(v[c]));
     }
-    const auto t = fx_fold_tables<N, N>(M);
+    const auto t = fx_fold_tables<N, N>(M, SYM, 60);
     unsigned mag = 0;
     for (int c = 0; c < N; ++c) mag = fx_mag(v[c]) > mag ? fx_mag(v[c]) : mag;
     if (fx_bad(mag)) std::exit(3);
@@ -41,7 +41,7 @@ static void lines(int spread, int shift) {
     for (int c = 0; c < N; ++c) fx_split(v[c], E, h[c], l[c]);
     double out[N];
     fx_contract<N, N, SYM>(t, h, l, [&](int k, long long R) {
-      if (R > (1ll << 61) || R < -(1ll << 61)) std::exit(4);
+      if (R > (1ll << 62) || R < -(1ll << 62)) std::exit(4);
       out[k] = fx_double(R, E - t.k);
     });
     for (int r = 0; r < N; ++r) {
