@@ -12,6 +12,7 @@
 // Schwarz, combined by a gather over the covering windows).
 #include <cmath>
 
+#include "fdm_window.h"
 #include "se_internal.h"
 
 namespace se {
@@ -194,27 +195,6 @@ int fdm_setup(const se_mesh_s* m, Level& lv, Allocs& allocs, bool want32, cudaSt
 }
 
 // ------------------------------------------------------------------ apply
-enum { FDM_RAS = 0, FDM_FULL = 1, FDM_EXT_IN = 2, FDM_GATHER = 3 };
-
-// Window point (a, b, c) of element e: neighbour slot and local index in that element.
-template <int P>
-__device__ __forceinline__ int64_t window_source(const int* __restrict__ nb, int64_t e, int a,
-                                                 int b, int c) {
-  constexpr int N = P + 1, PB = P + 3;
-  const int da = a == 0 ? -1 : (a == PB - 1 ? 1 : 0);
-  const int db = b == 0 ? -1 : (b == PB - 1 ? 1 : 0);
-  const int dc = c == 0 ? -1 : (c == PB - 1 ? 1 : 0);
-  int64_t src = e;
-  if (da | db | dc) {
-    src = nb[(da + 1) + 3 * (db + 1) + 9 * (dc + 1)];
-    if (src < 0) return -1;
-  }
-  const int ia = da < 0 ? P - 1 : (da > 0 ? 1 : a - 1);
-  const int ib = db < 0 ? P - 1 : (db > 0 ? 1 : b - 1);
-  const int ic = dc < 0 ? P - 1 : (dc > 0 ? 1 : c - 1);
-  return src * (N * N * N) + ia + N * (ib + N * ic);
-}
-
 // NE elements per block.  Each contraction phase gives one thread per line of every element
 // (lines numbered element-major), so active threads form a contiguous prefix and only the last
 // warp of a phase can be partly idle (one element per 128-thread block left 28 of 128 lanes
@@ -264,8 +244,8 @@ __device__ __forceinline__ T dot_row(const T* __restrict__ row, const T (&v)[PBP
   return acc;
 }
 
-// T is the arithmetic type (double, or df64: double-float on the FP32 pipe) and IO the type of
-// the vectors in memory (T, or double for df64).
+// T is the arithmetic type (df64: double-float on the FP32 pipe) and IO the type of the vectors in
+// memory (double).  T = double gathers windows only: the FP64 solves are fdm_fx_kernel's.
 template <int P, typename T, int MODE, typename IO = T>
 __global__ void __launch_bounds__(512) fdm_kernel(int64_t E, int NE, const int* __restrict__ nbr,
                                                   const IO* __restrict__ in,
@@ -1094,7 +1074,7 @@ size_t fdm_smem_bytes(int p, bool fp32, int ne) {
       per = fdm_smem_per_element<PP, float>();          \
       fixed = Fdm32Dims<PP + 3>::TAB_BYTES;             \
     } else {                                            \
-      per = fdm_smem_per_element<PP, double>();         \
+      per = fdm_fx_smem_per_element(PP);                \
     }                                                   \
     break;
     SE_FDM_SM(1) SE_FDM_SM(2) SE_FDM_SM(3) SE_FDM_SM(4) SE_FDM_SM(5)
@@ -1105,7 +1085,7 @@ size_t fdm_smem_bytes(int p, bool fp32, int ne) {
   return per * ne + fixed;
 }
 
-// Largest block: 256 threads for fdm32_warp_kernel (its launch bounds), 512 for fdm_kernel.
+// Largest block: 256 threads for fdm32_warp_kernel (its launch bounds), 512 in FP64 and df64.
 int fdm_max_threads(bool fp32) { return fp32 ? 256 : 512; }
 
 // Threads of a block with ne elements: FP32 one warp per element, FP64 one per line of a phase.
@@ -1115,15 +1095,19 @@ int fdm_block_threads(int p, bool fp32, int ne) {
 }
 
 // Elements per block: the tuned value if one is set and valid; else FP32 8 (one warp each),
-// FP64 about 400 lines per phase (at most 16 elements).
+// FP64 about 300 lines per phase (at most 16 elements).
 int fdm_elems_per_block(int p, bool fp32) {
   const int PB = p + 3;
   const int t = tile_get(p, fp32).fdm_ne;
   if (t >= 1 && t <= 16 && fdm_block_threads(p, fp32, t) <= fdm_max_threads(fp32) &&
       fdm_smem_bytes(p, fp32, t) <= 200 * 1024)
     return t;
-  int ne = fp32 ? 8 : 400 / (PB * PB);
-  ne = ne < 1 ? 1 : (ne > 16 ? 16 : ne);
+  // FP64 (fdm_fx_kernel), measured on GB300 (us per launch by elements per block): p = 3, 24^3:
+  // 2 78, 4 71, 6 67, 7 60; p = 5, 24^3: 1 174, 3 169, 4 166, 6 183; p = 6, 20^3: 1 188, 3 162, 4 188;
+  // p = 7, 24^3: 1 485, 2 424, 3 403, 4 442, 5 409; p = 8, 16^3: 1 193, 2 189, 3 181; p = 9, 16^3:
+  // 1 282, 2 263, 3 255; p = 10, 14^3: 1 256, 2 269, 3 250.  Blocks of about 300 lines
+  static const int ne64[SE_MAX_ORDER + 1] = {1, 16, 10, 7, 5, 4, 3, 3, 3, 3, 3};
+  int ne = fp32 ? 8 : ne64[p];
   while (ne > 1 && fdm_smem_bytes(p, fp32, ne) > 200 * 1024) --ne;
   return ne;
 }
@@ -1160,12 +1144,14 @@ static int launch_fdm(const Level& lv, const T* in, const T* S, const T* lam, T*
         fdm32_warp_kernel<P, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     SE_CUDA(attr);
     fdm32_warp_kernel<P, MODE><<<blocks, threads, smem, s>>>(lv.E, lv.nbr, in, S, lam, lv.pflag, out);
-  } else {
+  } else if constexpr (MODE == FDM_GATHER) {
     static const cudaError_t attr = cudaFuncSetAttribute(
         fdm_kernel<P, T, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     SE_CUDA(attr);
-    fdm_kernel<P, T, MODE><<<blocks, threads, smem, s>>>(lv.E, NE, lv.nbr, in, S, lam,
-                                                          lv.fdm_dinv64, lv.pflag, out);
+    fdm_kernel<P, T, MODE><<<blocks, threads, fdm_smem_per_element<P, T>() * NE, s>>>(
+        lv.E, NE, lv.nbr, in, S, lam, lv.fdm_dinv64, lv.pflag, out);
+  } else {
+    return fdm_fx_apply(lv, MODE, in, out, NE, s);
   }
   SE_LAUNCH_CHECK();
   return SE_OK;
@@ -1193,7 +1179,7 @@ template <int P, int MODE>
 static int launch_fdm_df(const Level& lv, const double* in, double* out, cudaStream_t s) {
   const int NE = fdm_df_elems_per_block(P);
   const int threads = fdm_block_threads(P, false, NE);
-  const size_t smem = fdm_smem_bytes(P, false, NE);
+  const size_t smem = fdm_smem_per_element<P, double>() * NE;
   const unsigned blocks = (unsigned)((lv.E + NE - 1) / NE);
   static const cudaError_t attr = cudaFuncSetAttribute(
       fdm_kernel<P, df64, MODE, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);

@@ -303,6 +303,10 @@ template <class T>
 int gather_ext(const Level& lv, const T* r, T* rbar, cudaStream_t s);
 template <class T>
 int fdm_apply_ext(const Level& lv, const T* rbar, T* zbar, cudaStream_t s);
+// FP64 solves in block floating point (fdm_fx.cu): mode FDM_RAS, FDM_FULL or FDM_EXT_IN, NE
+// elements per block.
+int fdm_fx_apply(const Level& lv, int mode, const double* in, double* out, int NE, cudaStream_t s);
+size_t fdm_fx_smem_per_element(int p);
 int fdm_setup(const se_mesh_s* m, Level& lv, Allocs& allocs, bool want32, cudaStream_t s,
               bool want_df = false);
 int asm_weights(Level& lv, Allocs& allocs, cudaStream_t s);

@@ -66,3 +66,58 @@ def test_operator_with_one_unscalable_value(p, value):
             assert np.max(np.abs(got[e] - ref[e])[ok[e]], initial=0.0) <= 1e-12 * scale + 5e-324, e
     finally:
         c.close()
+
+
+def _smoother(c, p, kind):
+    sched = (p, 1) if p < 4 else (p, p // 2, 1)
+    c.lv.extra["fdm"] = o.fdm_setup(c.lv, c.V, c.amp)
+    se = c.se
+    return se.se_pmg_setup(c.m, se.pmg_desc(sched, se.SE_SMOOTH_RAS if kind == "ras" else se.SE_SMOOTH_ASM, 1))
+
+
+@pytest.mark.parametrize("kind", ["ras", "asm"])
+@pytest.mark.parametrize("p", range(2, 11))
+def test_schwarz_blocks_and_range(p, kind):
+    """Element counts that leave a part of the last block empty; the residual scaled by powers of two
+    on both sides of the range of the common scale."""
+    c = Case((3, 3, 2) if p > 6 else (4, 3, 3), p, seed=80 + p, bc=("D", "D", "N", "D", "D", "N"))
+    try:
+        P = _smoother(c, p, kind)
+        r, s = c.random_continuous(5), c.empty()
+        ref = (o.ras if kind == "ras" else o.asm)(c.lv, r)
+        for k in (0, -985, -955, -800, 800, 990):
+            c.se.se_pmg_smooth(P, 0, c.to_gpu(np.ldexp(r, k)), s)
+            assert rel_err(np.ldexp(c.to_np(s), -k), ref) <= 1e-10, k
+        c.se.se_pmg_destroy(P)
+    finally:
+        c.close()
+
+
+@pytest.mark.parametrize("kind", ["ras", "asm"])
+@pytest.mark.parametrize("p,value", [(3, np.inf), (7, np.nan), (8, -np.inf)])
+def test_schwarz_with_one_unscalable_value(p, kind, value):
+    """The smoother is not finite exactly where the plain FP64 one is not; zeros stay zeros."""
+    c = Case((5, 3, 2), p, seed=7)
+    try:
+        P = _smoother(c, p, kind)
+        g = np.random.default_rng(3).uniform(-1, 1, c.lv.n_global)
+        g[c.lv.gid[0]] = 0.0
+        g[c.lv.gid[14, p // 2, p // 2, p // 2]] = value
+        r, s = o.from_global(c.lv, g), c.empty()
+        r = np.where(c.lv.mask > 0, r, 0.0)
+        with np.errstate(all="ignore"):
+            ref = (o.ras if kind == "ras" else o.asm)(c.lv, r)
+        ref = np.where(c.lv.mask > 0, ref, 0.0)
+        c.se.se_pmg_smooth(P, 0, c.to_gpu(r), s)
+        got = c.to_np(s)
+        ok = np.isfinite(ref)
+        assert not ok.all() and ok.any()
+        assert np.array_equal(np.isfinite(got)[c.lv.mask > 0], ok[c.lv.mask > 0])
+        scale = np.max(np.abs(ref[ok]))
+        both = ok & (c.lv.mask > 0)
+        assert np.max(np.abs(got[both] - ref[both])) <= 1e-10 * scale
+        c.se.se_pmg_smooth(P, 0, c.to_gpu(np.zeros_like(r)), s)
+        assert not c.to_np(s).any()
+        c.se.se_pmg_destroy(P)
+    finally:
+        c.close()
