@@ -310,7 +310,10 @@ size_t fdm_fx_smem_per_element(int p);
 int fdm_setup(const se_mesh_s* m, Level& lv, Allocs& allocs, bool want32, cudaStream_t s,
               bool want_df = false);
 int asm_weights(Level& lv, Allocs& allocs, cudaStream_t s);
-// Transfers (transfer.cu): level f (fine) <-> level c (coarse)
+// Transfers (transfer.cu): level f (fine) <-> level c (coarse); FP64 by transfer_fx (block floating
+// point, transfer_fx.cu), which leaves out the restriction's QQ^T
+int transfer_fx(const Level& f, const Level& c, bool restrict_, const double* J, const double* in, double* out,
+                bool accumulate, cudaStream_t s);
 template <class T>
 int restrict_apply(const Level& f, const Level& c, const T* J, const T* rf, T* rc,
                    cudaStream_t s);

@@ -2,23 +2,22 @@
 //   prolongation  e_f = (J x J x J) e_c            element by element
 //   restriction   r_c = M_c QQ^T_c (J^T x J^T x J^T)(r_f / mult_f)
 // with J_ij = h^c_j(xi^f_i).  For a continuous r_f the restriction is the transpose of the
-// global prolongation.  The three directions are contracted in turn through shared memory (the
-// folded kernel stores the last one straight from its lines).
+// global prolongation.  FP64 runs in transfer_fx.cu (block floating point); the kernels here are the
+// FP32 V-cycle's.  The three directions are contracted in turn through shared memory (the folded
+// kernel stores the last one straight from its lines).
 //
 // Both GLL node sets are symmetric about 0 and h^c_{Nc-1-j}(-x) = h^c_j(x), so J is
 // centro-symmetric: J[Nf-1-i][Nc-1-j] = J[i][j] (and so is J^T).  For even Nf and Nc each line
 // contraction runs folded (transfer_eo_kernel): with e_l = v_l + v_{n-1-l}, o_l = v_l - v_{n-1-l}
 // over the input line v of n points and Ep = (M[o][l] + M[o][n-1-l])/2, Om = (M[o][l] -
 // M[o][n-1-l])/2 for the line operator M (J or J^T), output o and its mirror are E_o + O_o and
-// E_o - O_o: n/2 fewer FMAs per output pair at the cost of n + m adds per line (about 20% fewer
-// FP64 instructions; GB300 runs this kernel on its FP64 pipe).  Several elements share a block.
-// At N = 4 <-> 2 the fold costs more than it saves (10 instead of 8 FP64 instructions per line):
-// transfer_small_kernel contracts densely, one thread per output value of each direction, several
-// elements per block.  Odd N (even orders) use the plain kernel, one element per block.
+// E_o - O_o: n/2 fewer FMAs per output pair at the cost of n + m adds per line.  Several elements
+// share a block.  At N = 4 <-> 2 the fold costs more than it saves (10 instead of 8 instructions per
+// line): transfer_small_kernel contracts densely, one thread per output value of each direction,
+// several elements per block.  Odd N (even orders) use the plain kernel, one element per block.
 // The restriction's 1/mult_f (1, 1/2, 1/4, 1/8) is applied by lowering the binary exponent with
-// integer instructions (scale_pow2), not by an FP64 multiply: exact for every value above 2^-1019
-// (2^-123 in FP32; smaller magnitudes, far below any residual a solve forms, become 0), and the
-// FP64 pipe keeps only the contractions.
+// integer instructions (scale_pow2): exact for every value above 2^-123 (2^-1019 in FP64; smaller
+// magnitudes, far below any residual a solve forms, become 0).
 #include "se_internal.h"
 #include "reduce.h"
 
@@ -318,7 +317,9 @@ int restrict_apply(const Level& f, const Level& c, const T* J, const T* rf, T* r
                    2.0 * f.E * (Nf * Nf * Nf * Nc + Nf * Nf * Nc * Nc + Nf * Nc * Nc * Nc),
                    prof_variant<T>(f.p));
     int st = SE_OK;
-    if (transfer_eo<T, true>(f, c, J, rf, f.pflag, rc, false, s, &st)) {
+    if constexpr (sizeof(T) == 8) {
+      SE_TRY(transfer_fx(f, c, true, J, rf, rc, false, s));
+    } else if (transfer_eo<T, true>(f, c, J, rf, f.pflag, rc, false, s, &st)) {
       SE_TRY(st);
     } else {
       transfer_kernel<T, true><<<(unsigned)f.E, 128, 0, s>>>(f.N, c.N, J, rf, f.pflag, rc, false);
@@ -336,6 +337,7 @@ int prolong_apply(const Level& f, const Level& c, const T* J, const T* ec, T* ef
                  f.E * (Nf * Nf * Nf * (accumulate ? 2.0 : 1.0) + Nc * Nc * Nc) * sizeof(T),
                  2.0 * f.E * (Nc * Nc * Nc * Nf + Nc * Nc * Nf * Nf + Nc * Nf * Nf * Nf),
                  prof_variant<T>(f.p));
+  if constexpr (sizeof(T) == 8) return transfer_fx(f, c, false, J, ec, ef, accumulate, s);
   int st = SE_OK;
   if (transfer_eo<T, false>(f, c, J, ec, nullptr, ef, accumulate, s, &st)) return st;
   transfer_kernel<T, false><<<(unsigned)f.E, 128, 0, s>>>(f.N, c.N, J, ec, nullptr, ef, accumulate);

@@ -63,7 +63,7 @@ def test_operator_with_one_unscalable_value(p, value):
         assert np.array_equal(np.isfinite(got), ok)
         for e in range(c.lv.E):
             scale = np.max(np.abs(ref[e][ok[e]]), initial=0.0)
-            assert np.max(np.abs(got[e] - ref[e])[ok[e]], initial=0.0) <= 1e-12 * scale + 5e-324, e
+            assert np.max(np.abs(got[e][ok[e]] - ref[e][ok[e]]), initial=0.0) <= 1e-12 * scale + 5e-324, e
     finally:
         c.close()
 
@@ -119,5 +119,38 @@ def test_schwarz_with_one_unscalable_value(p, kind, value):
         c.se.se_pmg_smooth(P, 0, c.to_gpu(np.zeros_like(r)), s)
         assert not c.to_np(s).any()
         c.se.se_pmg_destroy(P)
+    finally:
+        c.close()
+
+
+@pytest.mark.parametrize("pf,pc", [(2, 1), (4, 2), (7, 5), (8, 7), (9, 4), (10, 9), (10, 1)])
+def test_transfers_range_and_unscalable_values(pf, pc):
+    """Both transfers, scaled by powers of two on both sides of the range of the common scale, and with
+    one value that has no scale: not finite exactly where plain FP64 is not."""
+    c = Case((5, 3, 2), pf, seed=8)
+    try:
+        se = c.se
+        lc = o.make_level(c.V, c.nel, pc, c.lv.bc, c.amp)
+        P = se.se_pmg_setup(c.m, se.pmg_desc((pf, pc, 1) if pc > 1 else (pf, 1), se.SE_SMOOTH_JACOBI, 1))
+        rf, ec = c.random_continuous(6), c.random_continuous(7, lv=lc)
+        rc, ef = c.empty(lc.gid.size), c.empty()
+        ref_r, ref_e = o.restrict(c.lv, lc, rf), o.prolong(c.lv, lc, ec)
+        for k in (0, -1005, -955, 900, 1005):
+            se.se_pmg_restrict(P, 0, c.to_gpu(np.ldexp(rf, k)), rc)
+            se.se_pmg_prolong(P, 0, c.to_gpu(np.ldexp(ec, k)), ef)
+            assert rel_err(np.ldexp(rc.cpu().numpy().reshape(ref_r.shape), -k), ref_r) <= 1e-13, k
+            assert rel_err(np.ldexp(c.to_np(ef), -k), ref_e) <= 1e-13, k
+        for value in (np.inf, np.nan):
+            bad = ec.copy()
+            bad[7, 0, pc, 0] = value
+            se.se_pmg_prolong(P, 0, c.to_gpu(bad), ef)
+            with np.errstate(all="ignore"):
+                ref = o.prolong(c.lv, lc, bad)
+            ok = np.isfinite(ref)
+            got = c.to_np(ef)
+            # every value of the element depends on it (0 inf is NaN in plain FP64 too)
+            assert np.array_equal(np.isfinite(got), ok) and not ok[7].any() and ok[8].all()
+            assert np.max(np.abs(got[ok] - ref[ok])) <= 1e-13 * np.max(np.abs(ref[ok]))
+        se.se_pmg_destroy(P)
     finally:
         c.close()
