@@ -214,7 +214,8 @@ int ax_local(const Level& lv, const T* u, T* y, bool mask_in, cudaStream_t s, co
 //   y: lanes run along i: rows of N contiguous copies;
 //   z: lanes run along (i, j): planes of N^2 contiguous copies.
 // The y and z sweeps run as one launch (gs_sweep_yz): a node with copies across a y- and a
-// z-interface is summed by one thread in the order of the two sweeps.
+// z-interface is summed by one thread in the order of the two sweeps.  Small levels take one launch in
+// all (gs_all_kernel).
 // Masking (Dirichlet) zeroes the copies on Dirichlet faces within the x sweep, before any sum (a
 // node on such a face has all its copies there), so the sweeps then add zeros for masked nodes;
 // a lattice one element wide in x has a separate mask kernel.
@@ -430,6 +431,125 @@ __global__ void gs_mask_faces(int nx, int ny, int nz, int bits, T* __restrict__ 
   u[e * N3 + i + N * (j + N * k)] = T(0);
 }
 
+// Where one launch wins: a gathered x-face costs a sector per copy, so the sweeps move less data, but
+// they take two launches.  Measured on GB300 (us of se_gs, sweeps / one launch; FP64, back-to-back
+// launches): p = 7, 4^3 8.5 / 5.0, 8^3 9.7 / 6.6, 12^3 (0.9M points) 12.9 / 9.5, 16^3 (2.1M) 19.2 / 19.3,
+// 24^3 52 / 59, 32^3 114 / 133; p = 3, 16^3 (0.26M) 9.6 / 7.0, 24^3 (0.9M) 13.2 / 13.6, 32^3 19.4 / 22.6;
+// p = 1, 32^3 (0.26M) 12.6 / 8.5.  After the folded operator (fix-up and y/z launch against one): p = 7,
+// 4^3 23.0 / 19.8 with the operator, 12^3 41.3 / 38.9; p = 3, 24^3 36.4 / 39.0.
+constexpr int64_t GS_ONE_LAUNCH_POINTS = 600000;
+static bool gs_one_launch(const Level& lv) { return lv.L <= GS_ONE_LAUNCH_POINTS; }
+
+// QQ^T in one launch: a thread per point on an element's upper faces (i, j or k = p) whose copies the
+// element owns (no lower neighbour shares them) gathers the node's 2, 4 or 8 copies, sums them in the
+// order of the sweeps (x, then y, then z: the same bits) and writes the sum to all.  NE > 0: the x pairs
+// inside blocks of NE consecutive elements hold their sum already (the folded operator).  Dirichlet
+// nodes (bits) are left to threads of their own past the groups' (one per face copy), which write zeros.
+template <typename T, int N>
+__global__ void __launch_bounds__(256) gs_all_kernel(int nx, int ny, int nz, int NE, int bits, T* __restrict__ u) {
+  constexpr int N2 = N * N, N3 = N2 * N, P = N - 1, XI = N2, YI = N * P, ITEMS = N2 + N * P + P * P;
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  const unsigned groups = (unsigned)nx * ny * nz * ITEMS;
+  if (t >= groups) {
+    if (!bits) return;
+    unsigned r = t - groups;
+    const unsigned fx = (unsigned)ny * nz * N2, fy = (unsigned)nx * nz * N2, fz = (unsigned)nx * ny * N2;
+    int f;
+    if (r < 2 * fx) {
+      f = r < fx ? 0 : 1;
+      r -= f * fx;
+    } else if ((r -= 2 * fx) < 2 * fy) {
+      f = r < fy ? 2 : 3;
+      r -= (f - 2) * fy;
+    } else if ((r -= 2 * fy) < 2 * fz) {
+      f = r < fz ? 4 : 5;
+      r -= (f - 4) * fz;
+    } else {
+      return;
+    }
+    if (!((bits >> f) & 1)) return;
+    const int a = (int)(r % N), b = (int)((r / N) % N), el = (int)(r / N2), side = f & 1;
+    int ex, ey, ez, i, j, k;
+    if (f < 2) {
+      ey = el % ny; ez = el / ny; ex = side ? nx - 1 : 0;
+      i = side ? P : 0; j = a; k = b;
+    } else if (f < 4) {
+      ex = el % nx; ez = el / nx; ey = side ? ny - 1 : 0;
+      j = side ? P : 0; i = a; k = b;
+    } else {
+      ex = el % nx; ey = el / nx; ez = side ? nz - 1 : 0;
+      k = side ? P : 0; i = a; j = b;
+    }
+    u[(ex + nx * (ey + ny * ez)) * N3 + i + N * (j + N * k)] = T(0);
+    return;
+  }
+  // item: a point on an upper face of element e (its x-face, then the rest of its y-, then z-face)
+  const int e = (int)(t / ITEMS);
+  int q = (int)(t - (unsigned)e * ITEMS), i, j, k;
+  if (q < XI) {
+    i = P; j = q % N; k = q / N;
+  } else if ((q -= XI) < YI) {
+    j = P; i = q % P; k = q / P;
+  } else {
+    q -= YI;
+    k = P; i = q % P; j = q / P;
+  }
+  const int ex = e % nx, r2 = e / nx, ey = r2 % ny, ez = r2 / ny;
+  if ((i == 0 && ex > 0) || (j == 0 && ey > 0) || (k == 0 && ez > 0)) return;  // another element's
+  const bool x2 = i == P && ex < nx - 1, y2 = j == P && ey < ny - 1, z2 = k == P && ez < nz - 1;
+  if (((bits & 1) && i == 0 && ex == 0) || ((bits & 2) && i == P && ex == nx - 1) ||
+      ((bits & 4) && j == 0 && ey == 0) || ((bits & 8) && j == P && ey == ny - 1) ||
+      ((bits & 16) && k == 0 && ez == 0) || ((bits & 32) && k == P && ez == nz - 1))
+    return;
+  // rows of copies along x: (y, z) = (0, 0), (1, 0), (0, 1), (1, 1); a row's x pair may be summed already
+  const int dy = nx, dz = nx * ny;
+  int at[4];
+  T v[4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    at[r] = -1;
+    if ((!(r & 1) || y2) && (!(r & 2) || z2))
+      at[r] = (e + ((r & 1) ? dy : 0) + ((r & 2) ? dz : 0)) * N3 + i + N * ((r & 1) ? 0 : j) + N2 * ((r & 2) ? 0 : k);
+  }
+  bool pair[4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const int er = e + ((r & 1) ? dy : 0) + ((r & 2) ? dz : 0);
+    pair[r] = at[r] >= 0 && x2 && (NE == 0 || (er + 1) % NE == 0);
+  }
+  if (!y2 && !z2 && !pair[0]) return;  // nothing to add
+  T w[4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    v[r] = at[r] >= 0 ? u[at[r]] : T(0);
+    w[r] = pair[r] ? u[at[r] + N3 - P] : T(0);
+  }
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+    if (pair[r]) v[r] = v[r] + w[r];
+  T sum = y2 ? v[0] + v[1] : v[0];
+  if (z2) sum = sum + (y2 ? v[2] + v[3] : v[2]);
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+    if (at[r] >= 0) {
+      u[at[r]] = sum;
+      if (x2) u[at[r] + N3 - P] = sum;
+    }
+}
+
+
+template <typename T, int N>
+static int gs_all(const Level& lv, int NE, int bits, T* u, int var, double bytes, double flops, cudaStream_t s) {
+  const int nx = lv.nel[0], ny = lv.nel[1], nz = lv.nel[2];
+  constexpr int N2 = N * N, ITEMS = 3 * N2 - 3 * N + 1;
+  int64_t n = lv.E * ITEMS;
+  if (bits) n += 2 * N2 * ((int64_t)ny * nz + (int64_t)nx * nz + (int64_t)nx * ny);
+  ProfScope prof(SE_K_GS, s, (double)lv.L, bytes, flops, var);
+  gs_all_kernel<T, N><<<grid_for(n, 256), 256, 0, s>>>(nx, ny, nz, NE, bits, u);
+  SE_LAUNCH_CHECK();
+  return SE_OK;
+}
+
 // One profiling scope per launch (so launch counts are exact); the algorithmic bytes of QQ^T
 // (every interface copy read and written once) are attributed to the x sweep.
 template <typename T, int N>
@@ -441,6 +561,7 @@ static int gs_sweeps(const Level& lv, T* u, bool mask, double bytes, double flop
   if (mask)
     for (int f = 0; f < 6; ++f)
       if (lv.bc[f] == SE_BC_DIRICHLET) bits |= 1 << f;
+  if (gs_one_launch(lv)) return gs_all<T, N>(lv, 0, bits, u, var, bytes, flops, s);
   if (bits && nx == 1) {  // no x sweep to carry the mask
     {
       const int64_t n = 2 * N2 * ((int64_t)ny * nz + (int64_t)nx * nz + (int64_t)nx * ny);
@@ -501,6 +622,10 @@ static int gs_after_fold(const Level& lv, double* y, int NE, cudaStream_t s) {
   // the x direction must be complete before the y sweep adds across y-interfaces: a copy summed
   // across a block-boundary x-interface after the y sweep would count its y-partner's x-neighbour
   // twice
+  if (gs_one_launch(lv)) {
+    const double copies = yz_copies<N>(nx, ny, nz);
+    return gs_all<double, N>(lv, NE, 0, y, var, 2.0 * copies * sizeof(double), copies / 2, s);
+  }
   const int64_t nbnd = (lv.E + NE - 1) / NE - 1;
   if (nx > 1 && nbnd > 0) {
     const double n = (double)nbnd * N2;  // at most this many pairs

@@ -154,3 +154,26 @@ def test_transfers_range_and_unscalable_values(pf, pc):
         se.se_pmg_destroy(P)
     finally:
         c.close()
+
+
+@pytest.mark.parametrize("nel,p", [((1, 1, 1), 3), ((1, 4, 3), 2), ((5, 1, 2), 7), ((7, 6, 1), 4), ((9, 5, 4), 1),
+                                   ((30, 29, 31), 2), ((11, 12, 11), 7)])
+@pytest.mark.parametrize("bc", [("D",) * 6, ("N", "D", "D", "N", "N", "N")])
+def test_qqt_one_launch_and_sweeps(nel, p, bc):
+    """QQ^T with and without the mask on lattices one element wide in each direction, and on both sides
+    of the size where the one-launch form gives way to the sweeps; FP32 within one rounding per sum."""
+    c = Case(nel, p, seed=1, bc=bc)
+    try:
+        u = np.random.default_rng(4).uniform(-1, 1, c.lv.gid.shape)
+        for mask in (0, 1):
+            g = c.to_gpu(u)
+            c.se.se_gs(c.m, g, mask)
+            ref = o.qqt(c.lv, u)
+            if mask:
+                ref = c.lv.mask * ref
+            assert rel_err(c.to_np(g), ref) <= 1e-14
+        y = c.empty()
+        c.se.se_ax(c.m, c.to_gpu(u), y, c.se.SE_AX_ASSEMBLE | c.se.SE_AX_MASK | c.se.SE_AX_FP32)
+        assert rel_err(c.to_np(y), o.ax(c.lv, u)) <= 2e-5
+    finally:
+        c.close()
