@@ -22,12 +22,13 @@
 // left to gs_fold_fixup_x.
 //
 // Measured on GB300 (us per launch; in brackets the even-odd FP64 kernel this one replaced, which ran at
-// the FP64 pipe's 2 FMA/clk/SM): 32^3 elements p = 7 429 [1420], p = 5 196 [525], p = 3 57 [138]; even
-// orders (unfolded in FP64) 20^3 p = 8 192 [725].  Memory needs 158 us of the 429, the 9 FP64
-// instructions per point 240, and the integer pipes about the same: what is left are the waits between
-// them, so resident warps count (64 registers: 429, 80: 456, 96: 482; before the conversions back
-// were branch-free and G was prefetched to L2, 530 to 560).  u on the element's scale instead of each
-// line's was 4% faster, but lost accuracy where values within an element span many decades.
+// the FP64 pipe's 2 FMA/clk/SM): 32^3 elements p = 7 406 [1420], p = 5 198 [525], p = 3 54 [138]; even
+// orders (unfolded in FP64) 20^3 p = 8 182 [725].  Memory needs 158 us of the 406 and the 9 FP64
+// instructions per point 240; without both the kernel still takes 332: what bounds it is the issue of
+// about 430 instructions per 32 points, 72 of them multiply-adds of 3.5 cycles each.  64 registers beat
+// 48, 56, 72 and more; prefetching G to L2 costs more instructions than it saves waits.  u on the
+// element's scale instead of each line's was 4% faster, but lost accuracy where values within an
+// element span many decades.
 //
 // Error against extended precision (2-norm, on this repository's meshes), over that of the FP64 dot
 // products: 0.6 to 0.75 for random values, 0.3 to 0.8 for smooth ones, 0.6 for values that decay by
@@ -72,6 +73,25 @@ struct AxFxDims {
   static constexpr int NP = N % 2 ? N : N + 1;     // padded row: odd, so 8-byte lines do not conflict
   static constexpr int PLANE = NP * N, VOL = NP * N * N;
 };
+
+// A column's place in the lattice (FOLD): its element and its Dirichlet points (bit k).
+struct AxLattice {
+  int ex, ey, ez;
+  unsigned zmask;
+};
+template <int N>
+__device__ __forceinline__ AxLattice ax_lattice(const AxFxArgs& a, int e, int i, int j) {
+  AxLattice r;
+  r.ex = e % a.nx;
+  r.ey = (e / a.nx) % a.ny;
+  r.ez = e / (a.nx * a.ny);
+  const bool dxy = ((a.bits & 1) && i == 0 && r.ex == 0) || ((a.bits & 2) && i == N - 1 && r.ex == a.nx - 1) ||
+                   ((a.bits & 4) && j == 0 && r.ey == 0) || ((a.bits & 8) && j == N - 1 && r.ey == a.ny - 1);
+  r.zmask = dxy ? (1u << N) - 1u : 0u;
+  if ((a.bits & 16) && r.ez == 0) r.zmask |= 1u;
+  if ((a.bits & 32) && r.ez == a.nz - 1) r.zmask |= 1u << (N - 1);
+  return r;
+}
 
 // Input value of a local point: u, or D^-1 u, zero on masked points.
 __device__ __forceinline__ double ax_fx_input(const AxFxArgs& a, int64_t gi, bool zero) {
@@ -134,7 +154,7 @@ __device__ __noinline__ void ax_slow_block(const AxFxArgs& a, int64_t e, bool va
 // Registers: the kernel waits on memory, shared memory and dependent integer operations in turn, so
 // resident warps are worth more than registers up to the point where lines spill.
 template <int N>
-constexpr int ax_fx_regs() { return N <= 8 ? 64 : (N <= 10 ? 72 : 96); }
+constexpr int ax_fx_regs() { return N <= 9 ? 64 : (N == 10 ? 72 : 96); }
 
 template <int N, bool FOLD>
 __global__ void __maxnreg__(ax_fx_regs<N>())
@@ -154,27 +174,21 @@ __global__ void __maxnreg__(ax_fx_regs<N>())
   const int64_t eb = e * N3 + t;
   const int col = i + NP * j, rl = NP * i + PL * j, sl = i + PL * j;  // lines: column, (j=i,k=j), (i,k=j)
   if (t == 0) mags[le] = 0u;
-  // the geometric factors are needed after the forward contractions: on their way to L2 meanwhile
-  if (valid && t < 6 && N2 >= 6) fx_prefetch(a.G + t * a.L + e * N3, N3);
-  // Dirichlet points of the column (bit k)
-  unsigned zmask = 0u;
-  int ex = 0, ey = 0, ez = 0;
-  if constexpr (FOLD) {
-    const int ei = (int)e;  // E < 2^31
-    ex = ei % a.nx;
-    ey = (ei / a.nx) % a.ny;
-    ez = ei / (a.nx * a.ny);
-    const bool dxy = ((a.bits & 1) && i == 0 && ex == 0) || ((a.bits & 2) && i == N - 1 && ex == a.nx - 1) ||
-                     ((a.bits & 4) && j == 0 && ey == 0) || ((a.bits & 8) && j == N - 1 && ey == a.ny - 1);
-    if (dxy) zmask = (1u << N) - 1u;
-    if ((a.bits & 16) && ez == 0) zmask |= 1u;
-    if ((a.bits & 32) && ez == a.nz - 1) zmask |= 1u << (N - 1);
-  } else if (a.mask_in && valid) {
+  // the column's place in the lattice (E < 2^31): needed last, worth registers until then for small N
+  constexpr bool EARLY = FOLD && N < 8;
+  AxLattice at{};
+  if constexpr (EARLY) at = ax_lattice<N>(a, (int)e, i, j);
+  // Dirichlet points of the column (bit k), to mask the input
+  unsigned zin = 0u;
+  if (a.mask_in && valid) {
+    if constexpr (FOLD) {
+      zin = EARLY ? at.zmask : ax_lattice<N>(a, (int)e, i, j).zmask;
+    } else {
 #pragma unroll
-    for (int k = 0; k < N; ++k)
-      if (!(a.pflag[eb + N2 * k] & PF_FREE)) zmask |= 1u << k;
+      for (int k = 0; k < N; ++k)
+        if (!(a.pflag[eb + N2 * k] & PF_FREE)) zin |= 1u << k;
+    }
   }
-  const unsigned zin = a.mask_in ? zmask : 0u;
   bool bad = false;
   int Et;  // scale of the thread's column
   {
@@ -201,30 +215,42 @@ __global__ void __maxnreg__(ax_fx_regs<N>())
   }
   bad = __syncthreads_or(bad);
   if (!bad) {
-    // t-lines and the pointwise factors: the thread's column
+    // t-lines and the pointwise factors: the thread's column.  From N = 8 the factors have a loop of
+    // their own, two points at a time behind a barrier (which the compiler does not move loads across),
+    // so that the contraction and the loads in flight do not compete for registers: p = 7 429 -> 406 us,
+    // p = 8 192 -> 182, p = 9 283 -> 271; p = 5 and 6 are 8% faster fused (198, 138)
+    constexpr bool SPLIT = N >= 8;
+    unsigned mag = 0u;
+    const double* g = a.G + (valid ? eb : (int64_t)t);
+    auto pointwise = [&](int q, double ut) {
+      const double* gq = g + N2 * q;
+      const double grr = gq[0], grs = gq[a.L], grt = gq[2 * a.L], gss = gq[3 * a.L], gst = gq[4 * a.L], gtt = gq[5 * a.L];
+      const double ur = R[col + PL * q], us = S[col + PL * q];
+      const double wr = fma(grt, ut, fma(grs, us, grr * ur));
+      const double ws = fma(gst, ut, fma(gss, us, grs * ur));
+      const double wt = fma(gtt, ut, fma(gst, us, grt * ur));
+      R[col + PL * q] = wr;
+      S[col + PL * q] = ws;
+      U[col + PL * q] = wt;
+      mag = max(max(mag, fx_mag(wr)), max(fx_mag(ws), fx_mag(wt)));
+    };
     {
       const int eb1 = Et - tD.k;
       int h[N], l[N];
 #pragma unroll
       for (int q = 0; q < N; ++q) fx_split(U[col + PL * q], Et, h[q], l[q]);
-      unsigned mag = 0u;
       fx_contract<N, N, -1>(tD, h, l, [&](int q, long long r) {
-        const double ut = fx_double(r, eb1), ur = R[col + PL * q], us = S[col + PL * q];
-        double grr = 0.0, grs = 0.0, grt = 0.0, gss = 0.0, gst = 0.0, gtt = 0.0;
-        if (valid) {
-          const double* g = a.G + eb + N2 * q;
-          grr = g[0], grs = g[a.L], grt = g[2 * a.L], gss = g[3 * a.L], gst = g[4 * a.L], gtt = g[5 * a.L];
-        }
-        const double wr = fma(grt, ut, fma(grs, us, grr * ur));
-        const double ws = fma(gst, ut, fma(gss, us, grs * ur));
-        const double wt = fma(gtt, ut, fma(gst, us, grt * ur));
-        R[col + PL * q] = wr;
-        S[col + PL * q] = ws;
-        U[col + PL * q] = wt;
-        mag = max(max(mag, fx_mag(wr)), max(fx_mag(ws), fx_mag(wt)));
+        const double ut = fx_double(r, eb1);
+        if constexpr (SPLIT) U[col + PL * q] = ut;
+        else pointwise(q, ut);
       });
-      if (mag) atomicMax(&mags[le], mag);
     }
+    if constexpr (SPLIT) {
+      __syncthreads();
+#pragma unroll 2
+      for (int q = 0; q < N; ++q) pointwise(q, U[col + PL * q]);
+    }
+    if (mag) atomicMax(&mags[le], mag);
     __syncthreads();
     const unsigned mag2 = mags[le];
     const int E2 = fx_exponent(mag2);
@@ -258,12 +284,13 @@ __global__ void __maxnreg__(ax_fx_regs<N>())
     double yv[N];
 #pragma unroll
     for (int k = 0; k < N; ++k) yv[k] = U[col + PL * k];
+    if constexpr (!EARLY) at = ax_lattice<N>(a, (int)e, i, j);
     if (a.sub) {
-      const int xy = (int)((i == 0 && ex > 0) || (i == N - 1 && ex < a.nx - 1)) +
-                     (int)((j == 0 && ey > 0) || (j == N - 1 && ey < a.ny - 1));
+      const int xy = (int)((i == 0 && at.ex > 0) || (i == N - 1 && at.ex < a.nx - 1)) +
+                     (int)((j == 0 && at.ey > 0) || (j == N - 1 && at.ey < a.ny - 1));
 #pragma unroll
       for (int k = 0; k < N; ++k) {
-        const int zi = (int)((k == 0 && ez > 0) || (k == N - 1 && ez < a.nz - 1));
+        const int zi = (int)((k == 0 && at.ez > 0) || (k == N - 1 && at.ez < a.nz - 1));
         const double w = __longlong_as_double((long long)(1023 - xy - zi) << 52);
         yv[k] = valid ? a.sub[eb + N2 * k] * w - yv[k] : 0.0;
       }
@@ -271,8 +298,8 @@ __global__ void __maxnreg__(ax_fx_regs<N>())
     // x-interfaces inside the block: (N - 1, j, k) of element lp and (0, j, k) of lp + 1 when both
     // lie in one row; both copies get left + right.  Each pair is added once, by one lane of
     // densely packed warps (a warp-wide FP64 instruction costs the same with 2 or 32 lanes active)
-    const bool left = i == N - 1 && le + 1 < a.NE && e + 1 < a.E && ex < a.nx - 1;
-    const bool right = i == 0 && le > 0 && ex > 0;
+    const bool left = i == N - 1 && le + 1 < a.NE && e + 1 < a.E && at.ex < a.nx - 1;
+    const bool right = i == 0 && le > 0 && at.ex > 0;
     if (left || right) {
 #pragma unroll
       for (int k = 0; k < N; ++k) U[col + PL * k] = yv[k];
@@ -297,7 +324,7 @@ __global__ void __maxnreg__(ax_fx_regs<N>())
     }
     if (valid) {
 #pragma unroll
-      for (int k = 0; k < N; ++k) a.y[eb + N2 * k] = ((zmask >> k) & 1u) ? 0.0 : yv[k];
+      for (int k = 0; k < N; ++k) a.y[eb + N2 * k] = ((at.zmask >> k) & 1u) ? 0.0 : yv[k];
     }
   } else {
     if (valid) {
@@ -328,14 +355,22 @@ __global__ void gs_fold_fixup_x(int64_t E, int NE, int nx, double* __restrict__ 
 }
 
 template <int N>
+struct AxFxTables {
+  FxFold<N, N> D, T;  // three results of T = D^T are added in 64 bits
+  explicit AxFxTables(const double* d) : D(fx_fold_tables<N, N>(d, -1, 60)) {
+    double t[N * N];
+    for (int r = 0; r < N; ++r)
+      for (int c = 0; c < N; ++c) t[r * N + c] = d[c * N + r];
+    T = fx_fold_tables<N, N>(t, -1, 59);
+  }
+};
+
+template <int N>
 static int launch_ax_fx(const Level& lv, const double* u, double* y, bool mask_in, const double* sub,
                         const double* dinv, int NE, bool fold, cudaStream_t s) {
   static_assert(sizeof(FxFold<N, N>) <= 1536, "two folded tables and the arguments fit the 4 KB of parameters");
-  double Dt[N * N];
-  for (int r = 0; r < N; ++r)
-    for (int c = 0; c < N; ++c) Dt[r * N + c] = lv.basis.D[c * N + r];
-  // three results of D^T are added in 64 bits
-  const FxFold<N, N> tD = fx_fold_tables<N, N>(lv.basis.D, -1, 60), tT = fx_fold_tables<N, N>(Dt, -1, 59);
+  // the tables depend on the order only: formed once per process
+  static const AxFxTables<N> tab(lv.basis.D);
   AxFxArgs a{};
   a.E = lv.E;
   a.L = lv.L;
@@ -360,12 +395,12 @@ static int launch_ax_fx(const Level& lv, const double* u, double* y, bool mask_i
     static const cudaError_t attr = cudaFuncSetAttribute(
         ax_fx_kernel<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     SE_CUDA(attr);
-    ax_fx_kernel<N, true><<<blocks, threads, smem, s>>>(a, tD, tT);
+    ax_fx_kernel<N, true><<<blocks, threads, smem, s>>>(a, tab.D, tab.T);
   } else {
     static const cudaError_t attr = cudaFuncSetAttribute(
         ax_fx_kernel<N, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     SE_CUDA(attr);
-    ax_fx_kernel<N, false><<<blocks, threads, smem, s>>>(a, tD, tT);
+    ax_fx_kernel<N, false><<<blocks, threads, smem, s>>>(a, tab.D, tab.T);
   }
   SE_LAUNCH_CHECK();
   return SE_OK;
