@@ -48,13 +48,10 @@ enum se_status {
 };
 
 enum { SE_BC_DIRICHLET = 0, SE_BC_NEUMANN = 1 };
-/* Arithmetic of a preconditioner (se_pmg_desc.precision).  SE_DF64: FP64 vectors throughout, the
- * operator and FDM kernels of the smoothed levels compute in double-float arithmetic on the FP32
- * pipe (pairs of FP32 values, about 47-48 significant bits; odd orders use the even-odd folded
- * operator, even orders the plain sum factorisation).  Every df64 path (SE_DF64, SE_AX_DF64, operator_df64,
- * arnoldi_df64) takes operands of magnitude in [2^-103, 2^128) (about 1e-31 to 3e38) at that
- * accuracy; smaller values keep FP32 accuracy relative to themselves (below 2^-126 they are
- * zero) and larger ones overflow, so a problem scaled outside that range needs FP64. */
+/* Arithmetic of a preconditioner (se_pmg_desc.precision).  SE_DF64 (and SE_AX_DF64, operator_df64,
+ * arnoldi_df64 below) asked for double-float arithmetic, faster than the FP64 pipe at 47-48
+ * significant bits.  The FP64 kernels are now faster than that and exact to FP64 over its whole range,
+ * so all of these select them: SE_DF64 is SE_FP64 with problems kept out of a batch's groups. */
 enum { SE_FP64 = 0, SE_FP32 = 1, SE_DF64 = 2 };
 enum { SE_SMOOTH_JACOBI = 0, SE_SMOOTH_RAS = 1, SE_SMOOTH_ASM = 2 };
 enum { SE_FPCG = 0, SE_FGMRES = 1 };
@@ -116,8 +113,7 @@ int se_mesh_rhs(se_mesh_t m, const double* f_dev, double* b_dev, void* stream);
 /* ---------------------------------------------------------------- operator (Sec. 2.1) */
 /* y = [M] [QQ^T] A_L [M] u.  flags: SE_AX_ASSEMBLE applies QQ^T (direct stiffness
  * summation), SE_AX_MASK zeroes Dirichlet nodes of input and output, SE_AX_FP32 computes in
- * FP32, SE_AX_DF64 in double-float arithmetic (the first call
- * allocates df64 copies of the geometric factors, 6 L x 8 bytes, owned by the mesh); inputs and
+ * FP32 (SE_AX_DF64: as without it); inputs and
  * outputs stay FP64.  A_L is applied by tensor-product sum factorisation
  * (Sec. 1: ~7E(p+1)^3 reads, 12E(p+1)^4 operations).  u and y must not overlap. */
 int se_ax(se_mesh_t m, const double* u, double* y, int flags, void* stream);
@@ -177,12 +173,9 @@ typedef struct se_pmg_desc {
   double coarse_tol;             /* coarsest-level Jacobi-PCG relative tolerance (1e-2) */
   int coarse_maxit;              /* and iteration cap (500) */
   int precision;                 /* SE_FP64; SE_FP32 for the whole V-cycle except the coarse
-                                    solve (Arnoldi and coarse solve stay FP64); SE_DF64: FP64
-                                    vectors, operator and FDM kernels in double-float */
-  int arnoldi_df64;              /* 1: the Arnoldi rounds of an SE_FP64 or SE_FP32 preconditioner
-                                    apply the operator and FDM kernels in double-float (FP64
-                                    vectors; df64 copies of the level data exist
-                                    only during the set-up).  SE_DF64 always does. */
+                                    solve (Arnoldi and coarse solve stay FP64); SE_DF64: as
+                                    SE_FP64 */
+  int arnoldi_df64;              /* 0 or 1: no effect (the Arnoldi rounds are FP64) */
   int cycle;                     /* SE_CYCLE_MULTIPLICATIVE (0): Algorithm 1 with the Chebyshev
                                     smoother.  SE_CYCLE_ADDITIVE (1): the additive V-cycle the
                                     paper uses for Schwarz smoothers without Chebyshev
@@ -263,8 +256,7 @@ typedef struct se_solve_opts {
   int tol_norm;      /* SE_TOL_R0 (0): stop when ||r_k|| <= tol ||r_0||; SE_TOL_B (1): when
                         ||r_k|| <= tol ||b|| (for an initial guess from se_proj_guess: the same
                         accuracy whatever the guess; 0 iterations if the guess already meets it) */
-  int operator_df64; /* 1: the outer operator A x computes in double-float arithmetic, as se_ax
-                        with SE_AX_DF64 */
+  int operator_df64; /* 0 or 1: no effect (the outer operator is FP64) */
 } se_solve_opts;
 enum { SE_TOL_R0 = 0, SE_TOL_B = 1 };
 
@@ -433,8 +425,7 @@ typedef struct se_serve_cfg {
                               projection space of that many prior solutions (se_proj_*), a
                               request on it starts from the projected guess and stops when
                               ||r|| <= tol ||b|| (counted in the footprint) */
-  int operator_df64;       /* 1: outer operators of resident meshes compute in double-float
-                              (df64 copies of the geometry, 48 bytes per point, counted) */
+  int operator_df64;       /* 0 or 1: no effect (outer operators are FP64) */
 } se_serve_cfg;
 typedef struct se_serve_stats {
   int64_t submitted, completed, refused, failed, pending;

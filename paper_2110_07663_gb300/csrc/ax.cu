@@ -9,15 +9,15 @@ namespace se {
 //   ur = D_r u, us = D_s u, ut = D_t u         (the t contraction runs in registers)
 //   (wr, ws, wt) = G (ur, us, ut), G symmetric with 6 stored factors per point
 //   y = D_r^T wr + D_s^T ws + D_t^T wt         (the t part accumulates in registers)
-// 12N+15 flops per point; reads u and G (7 values) and writes y once.  T is the arithmetic type,
-// IO the type of u, y and sub in memory (T, or double for T = df64).
-template <int N, typename T, typename IO = T>
-__global__ void __launch_bounds__(512) ax_local_kernel(int64_t E, int NE, const IO* __restrict__ u,
+// 12N+15 flops per point; reads u and G (7 values) and writes y once.  FP32: odd N, and even N with
+// an input mask (the rest is ax_tma.cu's; FP64 is ax_fx.cu's).
+template <int N, typename T>
+__global__ void __launch_bounds__(512) ax_local_kernel(int64_t E, int NE, const T* __restrict__ u,
                                                        const T* __restrict__ G, int64_t L,
                                                        const T* __restrict__ Dg,
-                                                       IO* __restrict__ y,
+                                                       T* __restrict__ y,
                                                        const uint8_t* __restrict__ pflag,
-                                                       bool mask_in, const IO* __restrict__ sub) {
+                                                       bool mask_in, const T* __restrict__ sub) {
   constexpr int N2 = N * N, N3 = N * N * N;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* sD = reinterpret_cast<T*>(smem_raw);
@@ -36,7 +36,7 @@ __global__ void __launch_bounds__(512) ax_local_kernel(int64_t E, int NE, const 
   for (int k = 0; k < N; ++k) {
     T v = T(0);
     if (valid) {
-      v = from_io<T>(u[eb + ij + N2 * k]);
+      v = u[eb + ij + N2 * k];
       if (mask_in && !(pflag[eb + ij + N2 * k] & PF_FREE)) v = T(0);
     }
     ru[k] = v;
@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(512) ax_local_kernel(int64_t E, int NE, const 
       acc += Dci[l] * swr[l + N * j + N2 * k];
       acc += Dcj[l] * sws[i + N * l + N2 * k];
     }
-    if (valid) y[eb + ij + N2 * k] = ax_output(io_cast<IO>(acc), sub, pflag, eb + ij + N2 * k);
+    if (valid) y[eb + ij + N2 * k] = ax_output(acc, sub, pflag, eb + ij + N2 * k);
   }
 }
 
@@ -137,36 +137,6 @@ static int launch_ax(const Level& lv, const T* u, T* y, const T* G, const T* D, 
   return SE_OK;
 }
 
-// df64 arithmetic on FP64 vectors, odd N (even orders; even N uses the folded kernel).
-template <int N>
-static int launch_ax_df(const Level& lv, const double* u, double* y, const double* sub,
-                        cudaStream_t s) {
-  const int NE = ax_elems_per_block(N - 1, false);
-  const int threads = NE * N * N;
-  const size_t smem = (N * N + (size_t)NE * 3 * N * N * N) * sizeof(df64);
-  static const cudaError_t attr = cudaFuncSetAttribute(
-      ax_local_kernel<N, df64, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-  SE_CUDA(attr);
-  const unsigned blocks = (unsigned)((lv.E + NE - 1) / NE);
-  ax_local_kernel<N, df64, double><<<blocks, threads, smem, s>>>(lv.E, NE, u, lv.Gdf, lv.L, lv.Ddf, y,
-                                                                  lv.pflag, false, sub);
-  SE_LAUNCH_CHECK();
-  return SE_OK;
-}
-
-static int ax_local_generic_df(const Level& lv, const double* u, double* y, const double* sub,
-                               cudaStream_t s) {
-  SE_CHECK(lv.Gdf != nullptr && lv.Ddf != nullptr, SE_EINVAL, "ax_df: df64 geometry missing");
-  switch (lv.N) {
-    case 3: return launch_ax_df<3>(lv, u, y, sub, s);
-    case 5: return launch_ax_df<5>(lv, u, y, sub, s);
-    case 7: return launch_ax_df<7>(lv, u, y, sub, s);
-    case 9: return launch_ax_df<9>(lv, u, y, sub, s);
-    case 11: return launch_ax_df<11>(lv, u, y, sub, s);
-    default: set_error("ax_df: unsupported N=%d", lv.N); return SE_EINVAL;
-  }
-}
-
 template <class T>
 int ax_local(const Level& lv, const T* u, T* y, bool mask_in, cudaStream_t s, const T* sub) {
   const void* G;
@@ -175,17 +145,11 @@ int ax_local(const Level& lv, const T* u, T* y, bool mask_in, cudaStream_t s, co
   SE_CHECK(G != nullptr, SE_EINVAL, "ax_local: geometric factors for this precision missing");
   const int N = lv.N;
   const double pts = (double)lv.L;
-  bool use_df = false;
-  if constexpr (sizeof(T) == 8) use_df = !mask_in && ax_df_route(lv);
   ProfScope prof(SE_K_AX, s, pts, pts * ((sub ? 9.0 : 8.0) * sizeof(T) + (sub ? 1.0 : 0.0)),
-                 pts * (12.0 * N + 15.0), use_df ? lv.p + 64 : prof_variant<T>(lv.p));
+                 pts * (12.0 * N + 15.0), prof_variant<T>(lv.p));
   if constexpr (sizeof(T) == 4) {
     if (!mask_in && ax_tma_supported(lv.p)) return ax_local_tma(lv, u, y, s, sub);
   } else {
-    if (use_df) {
-      if (ax_eo_supported(lv.p)) return ax_local_eo_df(lv, u, y, s, sub);
-      return ax_local_generic_df(lv, u, y, sub, s);
-    }
     return ax_local_fx(lv, u, y, mask_in, sub, nullptr, ax_elems_per_block(lv.p, false), false, s);
   }
   if constexpr (sizeof(T) == 4) {
@@ -611,7 +575,7 @@ int gs_apply(const Level& lv, T* u, bool mask, cudaStream_t s) {
 // reads and writes every sector of the vector (an x-interface copy is the first or last value of
 // a row of N), from the operator applications of the solve.
 bool ax_fold_ok(const Level& lv) {
-  return !ax_df_route(lv) && !lv.gsm_ids && lv.nel[0] >= 1 && lv.nel[1] >= 1 && lv.nel[2] >= 1;
+  return !lv.gsm_ids && lv.nel[0] >= 1 && lv.nel[1] >= 1 && lv.nel[2] >= 1;
 }
 
 template <int N>
@@ -696,21 +660,6 @@ int se_ax(se_mesh_t m, const double* u, double* y, int flags, void* stream) {
     if (!assemble && mask) SE_TRY(apply_mask64(lv, y, s));
     return SE_OK;
   }
-  if (flags & SE_AX_DF64) {
-    SE_TRY(make_df_geometry(lv, m->allocs, s));
-    Level ld = lv;
-    ld.df = true;
-    const double* in = u;
-    if (mask) {  // masked input through the mesh's work vector
-      SE_CUDA(cudaMemcpyAsync(m->tmp64, u, lv.L * sizeof(double), cudaMemcpyDeviceToDevice, s));
-      SE_TRY(apply_mask64(lv, m->tmp64, s));
-      in = m->tmp64;
-    }
-    SE_TRY(ax_local<double>(ld, in, y, false, s));
-    if (assemble) return gs_apply<double>(ld, y, mask, s);
-    if (mask) return apply_mask64(lv, y, s);
-    return SE_OK;
-  }
   if (assemble && mask && ax_fold_ok(lv)) return ax_apply_folded(lv, u, y, nullptr, s, nullptr, true);
   SE_TRY(ax_local<double>(lv, u, y, mask, s));
   if (assemble) return gs_apply<double>(lv, y, mask, s);
@@ -732,12 +681,6 @@ int se_residual(se_mesh_t m, const double* b, const double* u, double* r, int fl
     SE_TRY((convert<double, float>(b, m->tmpc32, lv.L, s)));
     SE_TRY(residual_apply<float>(lv, m->tmpc32, m->tmpa32, m->tmpb32, s));
     return convert<float, double>(m->tmpb32, r, lv.L, s);
-  }
-  if (flags & SE_AX_DF64) {
-    SE_TRY(make_df_geometry(lv, m->allocs, s));
-    Level ld = lv;
-    ld.df = true;
-    return residual_apply<double>(ld, b, u, r, s);
   }
   return residual_apply<double>(lv, b, u, r, s);
 }

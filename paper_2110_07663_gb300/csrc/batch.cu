@@ -371,7 +371,6 @@ static int build_union_level(se_pmg_s* U, int l, const std::vector<se_pmg_s*>& P
   u.basis = a0.basis;
   u.D64 = a0.D64;   // derivative tables depend on p only: shared with member 0
   u.D32 = a0.D32;
-  u.eo64 = a0.eo64;
   for (int f = 0; f < 6; ++f) u.bc[f] = a0.bc[f];
   for (const se_pmg_s* P : Pm) {
     u.E += P->lv[l]->E;
@@ -494,7 +493,7 @@ static void destroy_group(BatchGroup* G) {
   delete G;
 }
 
-static int build_group(BatchGroup* G, const std::vector<se_problem>& probs, int op_df) {
+static int build_group(BatchGroup* G, const std::vector<se_problem>& probs) {
   const int n = G->n = (int)G->idx.size();
   std::vector<se_pmg_s*> Pm(n);
   for (int m = 0; m < n; ++m) Pm[m] = probs[G->idx[m]].pmg;
@@ -536,11 +535,8 @@ static int build_group(BatchGroup* G, const std::vector<se_problem>& probs, int 
   SE_TRY(coarse_group_setup(&G->cg, clv.data(), cwk.data(), n, fp32, rin, xout, coff.data(),
                             d.coarse_tol, d.coarse_maxit, U->allocs, s));
   U->cgroup = &G->cg;
-  // outer solver state: level 0 in FP64, or in double-float arithmetic (operator_df64; the df64
-  // geometry is made for the outer operator only, the V-cycle keeps its own arithmetic)
-  if (op_df) SE_TRY(make_df_geometry(U->owned[0], U->allocs, s));
+  // outer solver state: level 0 in FP64
   G->fine = U->owned[0];
-  G->fine.df = op_df != 0;
   const int64_t L = G->fine.L;
   Allocs& A = U->allocs;
   for (double** v : {&G->b, &G->x, &G->r, &G->r_old, &G->z, &G->p, &G->w}) SE_TRY(dmalloc(A, v, (size_t)L));
@@ -809,13 +805,11 @@ int se_batch_create(int n, const se_problem* probs, const se_solve_opts* opts, s
     auto* G = new BatchGroup();
     G->idx = members[g];
     B->groups.push_back(G);
-    rc = build_group(G, B->probs, opts->operator_df64);
+    rc = build_group(G, B->probs);
   }
   for (int i : B->alone) {
     if (rc != SE_OK) break;
     rc = prepare_graph_solve(probs[i].mesh);
-    if (rc == SE_OK && opts->operator_df64)
-      rc = make_df_geometry(probs[i].mesh->fine, probs[i].mesh->allocs, probs[i].mesh->stream);
   }
   B->host = opts->graph_capture == 0;
   B->alone_stats.assign(n, se_solve_stats{});
@@ -844,7 +838,7 @@ int se_batch_create(int n, const se_problem* probs, const se_solve_opts* opts, s
   for (int i : B->alone) {
     if (rc != SE_OK) break;
     rc = append_fpcg_solve(Gr, cs, probs[i].mesh, probs[i].pmg, probs[i].b, probs[i].x, opts->tol,
-                           opts->maxit, opts->tol_norm, opts->operator_df64);
+                           opts->maxit, opts->tol_norm);
   }
   if (cs) cudaStreamDestroy(cs);
   if (rc == SE_OK && cudaGraphInstantiate(&B->exec, Gr, 0) != cudaSuccess) {

@@ -147,8 +147,7 @@ __global__ void cast_kernel(int64_t n, const double* __restrict__ a, T* __restri
   if (i < n) b[i] = (T)a[i];
 }
 
-int fdm_setup(const se_mesh_s* m, Level& lv, Allocs& allocs, bool want32, cudaStream_t s,
-              bool want_df) {
+int fdm_setup(const se_mesh_s* m, Level& lv, Allocs& allocs, bool want32, cudaStream_t s) {
   const int P = lv.p, N = P + 1, PB = P + 3;
   const int64_t E = lv.E;
   // 1D GLL stiffness D^T W D (reference element)
@@ -185,239 +184,22 @@ int fdm_setup(const se_mesh_s* m, Level& lv, Allocs& allocs, bool want32, cudaSt
     cast_kernel<float><<<grid_for(3 * E * PB, 256), 256, 0, s>>>(3 * E * PB, lv.lam64, lv.lam32);
     SE_LAUNCH_CHECK();
   }
-  if (want_df) {
-    SE_TRY(dmalloc(allocs, &lv.Sdf, 3 * E * PB * PB));
-    SE_TRY(dmalloc(allocs, &lv.lamdf, 3 * E * PB));
-    SE_TRY(split_df(lv.S64, lv.Sdf, 3 * E * PB * PB, s));
-    SE_TRY(split_df(lv.lam64, lv.lamdf, 3 * E * PB, s));
-  }
   return SE_OK;
 }
 
 // ------------------------------------------------------------------ apply
-// NE elements per block.  Each contraction phase gives one thread per line of every element
-// (lines numbered element-major), so active threads form a contiguous prefix and only the last
-// warp of a phase can be partly idle (one element per 128-thread block left 28 of 128 lanes
-// idle at p = 7).  S and S^T sit in shared memory with rows padded to a multiple of 4 entries
-// and are read as 16-byte vectors (4 FP32 or 2 FP64 values per load) against register lines
-// padded with zeros: the forward transform uses rows of S^T, the backward one rows of S.
-template <int PB>
-struct FdmDims {
-  static constexpr int PBP = (PB + 3) / 4 * 4;            // padded row length
-  static constexpr int PB3 = PB * PB * PB;
-  static constexpr int PB3P = (PB3 + 3) / 4 * 4;           // buffer length, 16-byte multiple
-  static constexpr int SROW = 3 * PB * PBP;                // S or S^T of 3 directions
-};
-
-// One FMA per multiply-add.  FP32: 16-byte loads of the padded row (the FP32 kernel is not
-// ALU-bound; padding entries are zero).  FP64 (ALU-bound): scalar loads of the PB real entries.
-template <int PB, int PBP, typename T>
-__device__ __forceinline__ T dot_row(const T* __restrict__ row, const T (&v)[PBP]) {
-  T acc = T(0);
-  if constexpr (sizeof(T) == 4) {
-#pragma unroll
-    for (int a = 0; a < PBP; a += 4) {
-      const float4 s = *reinterpret_cast<const float4*>(row + a);
-      acc = fmaf(s.x, v[a], acc);
-      acc = fmaf(s.y, v[a + 1], acc);
-      acc = fmaf(s.z, v[a + 2], acc);
-      acc = fmaf(s.w, v[a + 3], acc);
-    }
-  } else if constexpr (is_df64<T>::value) {
-    // two independent accumulation chains (a df64 product-accumulate is a chain of about 10
-    // dependent FP32 operations, so one chain per row would leave the FP32 pipe waiting on
-    // latency), renormalised once at the end
-    df_acc A0, A1;
-#pragma unroll
-    for (int a = 0; a + 1 < PB; a += 2) {
-      // rows are padded to PBP (a multiple of 4) entries: two df64 values per 16-byte load
-      const float4 q = *reinterpret_cast<const float4*>(row + a);
-      df_acc_fma(A0, df64(q.x, q.y), v[a]);
-      df_acc_fma(A1, df64(q.z, q.w), v[a + 1]);
-    }
-    if constexpr (PB % 2 == 1) df_acc_fma(A0, row[PB - 1], v[PB - 1]);
-    acc = df_acc_merge(A0, A1);
-  } else {
-#pragma unroll
-    for (int a = 0; a < PB; ++a) acc = fma(row[a], v[a], acc);
-  }
-  return acc;
-}
-
-// T is the arithmetic type (df64: double-float on the FP32 pipe) and IO the type of the vectors in
-// memory (double).  T = double gathers windows only: the FP64 solves are fdm_fx_kernel's.
-template <int P, typename T, int MODE, typename IO = T>
-__global__ void __launch_bounds__(512) fdm_kernel(int64_t E, int NE, const int* __restrict__ nbr,
-                                                  const IO* __restrict__ in,
-                                                  const T* __restrict__ Sg,
-                                                  const T* __restrict__ lamg,
-                                                  const double* __restrict__ dinvg,
-                                                  const uint8_t* __restrict__ pflag,
-                                                  IO* __restrict__ out) {
-  constexpr int N = P + 1, PB = P + 3, PB2 = PB * PB, PB3 = PB * PB * PB;
-  using Dm = FdmDims<PB>;
-  constexpr int PBP = Dm::PBP, PB3P = Dm::PB3P, SROW = Dm::SROW;
-  constexpr int LAMP = (3 * PB + 3) / 4 * 4;
-  constexpr int PER = 2 * PB3P + 2 * SROW + LAMP;  // shared values per element
-  // output loops: fully unrolled in FP64; df64 unrolls them twice only (a df64 row dot product
-  // is about 150 instructions, and the fully unrolled kernel overflows the instruction cache)
-  constexpr int OUT_UNR = is_df64<T>::value ? 2 : PB;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* sbase = reinterpret_cast<T*>(smem_raw);
-  int* snb = reinterpret_cast<int*>(sbase + (size_t)NE * PER);  // [NE][27]
-  const int64_t e0 = (int64_t)blockIdx.x * NE;
-  const int ne = (int)((E - e0) < NE ? (E - e0) : NE);             // elements in this block
-  const int tid = threadIdx.x, nt = blockDim.x;
-  auto B0 = [&](int le) { return sbase + (size_t)le * PER; };
-  auto B1 = [&](int le) { return sbase + (size_t)le * PER + PB3P; };
-  auto ST = [&](int le) { return sbase + (size_t)le * PER + 2 * PB3P; };          // S^T rows
-  auto SR = [&](int le) { return sbase + (size_t)le * PER + 2 * PB3P + SROW; };   // S rows
-  auto SL = [&](int le) { return sbase + (size_t)le * PER + 2 * PB3P + 2 * SROW; };
-  if constexpr (MODE != FDM_GATHER) {
-    // S[d][row][col] (row = window point, col = mode) -> S^T[d][col][row], S[d][row][col], padded
-    for (int q = tid; q < ne * 3 * PB * PBP; q += nt) {
-      const int le = q / (3 * PB * PBP), r = q - le * 3 * PB * PBP;
-      const int d = r / (PB * PBP), rr = r - d * PB * PBP;
-      const int i = rr / PBP, j = rr - i * PBP;
-      const T* S = Sg + ((e0 + le) * 3 + d) * PB2;
-      ST(le)[r] = j < PB ? S[j * PB + i] : T(0);
-      SR(le)[r] = j < PB ? S[i * PB + j] : T(0);
-    }
-    for (int q = tid; q < ne * 3 * PB; q += nt) {
-      const int le = q / (3 * PB), r = q - le * 3 * PB;
-      SL(le)[r] = lamg[(e0 + le) * 3 * PB + r];
-    }
-  }
-  for (int q = tid; q < ne * 27; q += nt) snb[q] = nbr[27 * e0 + q];
-  __syncthreads();
-  // ---- gather the extended window: one thread per (element, a, b), loop over c
-  if constexpr (MODE == FDM_EXT_IN) {
-    for (int q = tid; q < ne * PB3; q += nt) {
-      const int le = q / PB3;
-      B0(le)[q - le * PB3] = from_io<T>(in[e0 * PB3 + q]);
-    }
-  } else {
-    if (tid < ne * PB2) {
-      const int le = tid / PB2, ql = tid - le * PB2;
-      const int a = ql % PB, b = ql / PB;
-      T* b0 = B0(le);
-      for (int c = 0; c < PB; ++c) {
-        const int64_t src = window_source<P>(snb + 27 * le, e0 + le, a, b, c);
-        b0[a + PB * (b + PB * c)] = src >= 0 ? from_io<T>(in[src]) : T(0);
-      }
-    }
-  }
-  if constexpr (MODE == FDM_GATHER) {
-    __syncthreads();
-    for (int q = tid; q < ne * PB3; q += nt) {
-      const int le = q / PB3;
-      out[e0 * PB3 + q] = io_cast<IO>(B0(le)[q - le * PB3]);
-    }
-    return;
-  } else {
-    __syncthreads();
-    T v[PBP];
-#pragma unroll
-    for (int a = PB; a < PBP; ++a) v[a] = T(0);
-    const bool full_line = tid < ne * PB2;
-    const int le = full_line ? tid / PB2 : 0;
-    const int ql = tid - le * PB2;
-    const T* STx = ST(le);
-    const T* STy = STx + PB * PBP;
-    const T* STz = STx + 2 * PB * PBP;
-    const T* SRz = SR(le) + 2 * PB * PBP;
-    const T* sl = SL(le);
-    T* b0 = B0(le);
-    T* b1 = B1(le);
-    // ---- forward: S_x^T along a (line (b, c))
-    if (full_line) {
-      const int b = ql % PB, c = ql / PB;
-#pragma unroll
-      for (int a = 0; a < PB; ++a) v[a] = b0[a + PB * (b + PB * c)];
-#pragma unroll OUT_UNR
-      for (int al = 0; al < PB; ++al) b1[al + PB * (b + PB * c)] = dot_row<PB, PBP>(STx + al * PBP, v);
-    }
-    __syncthreads();
-    // ---- forward: S_y^T along b (line (alpha, c))
-    if (full_line) {
-      const int al = ql % PB, c = ql / PB;
-#pragma unroll
-      for (int b = 0; b < PB; ++b) v[b] = b1[al + PB * (b + PB * c)];
-#pragma unroll OUT_UNR
-      for (int be = 0; be < PB; ++be) b0[al + PB * (be + PB * c)] = dot_row<PB, PBP>(STy + be * PBP, v);
-    }
-    __syncthreads();
-    // ---- forward: S_z^T along c, then D^-1 (line (alpha, beta))
-    if (full_line) {
-      const int al = ql % PB, be = ql / PB;
-#pragma unroll
-      for (int c = 0; c < PB; ++c) v[c] = b0[al + PB * (be + PB * c)];
-      const T lxy = sl[al] + sl[PB + be];
-#pragma unroll OUT_UNR
-      for (int ga = 0; ga < PB; ++ga) {
-        const T acc = dot_row<PB, PBP>(STz + ga * PBP, v);
-        const int q = al + PB * (be + PB * ga);
-        T dv;
-        if constexpr (sizeof(T) == 8) dv = from_io<T>(dinvg[(e0 + le) * PB3 + q]);
-        else dv = __frcp_rn(lxy + sl[2 * PB + ga]);
-        b1[q] = acc * dv;
-      }
-    }
-    __syncthreads();
-    // ---- backward: S_z along gamma (own outputs c' = 1..N for RAS, all PB otherwise)
-    constexpr int C0 = MODE == FDM_RAS ? 1 : 0;
-    constexpr int NC = MODE == FDM_RAS ? N : PB;
-    if (full_line) {
-      const int al = ql % PB, be = ql / PB;
-#pragma unroll
-      for (int ga = 0; ga < PB; ++ga) v[ga] = b1[al + PB * (be + PB * ga)];
-#pragma unroll OUT_UNR
-      for (int cc = 0; cc < NC; ++cc) {
-        const int c = C0 + cc;
-        b0[al + PB * (be + PB * c)] = dot_row<PB, PBP>(SRz + c * PBP, v);
-      }
-    }
-    __syncthreads();
-    // ---- backward: S_y along beta (line (alpha, c'), PB*NC lines per element)
-    if (tid < ne * PB * NC) {
-      const int le2 = tid / (PB * NC), q2 = tid - le2 * PB * NC;
-      const int al = q2 % PB, c = C0 + q2 / PB;
-      const T* SRy = SR(le2) + PB * PBP;
-      T* b0e = B0(le2);
-      T* b1e = B1(le2);
-#pragma unroll
-      for (int be = 0; be < PB; ++be) v[be] = b0e[al + PB * (be + PB * c)];
-#pragma unroll OUT_UNR
-      for (int bb = 0; bb < NC; ++bb) {
-        const int b = C0 + bb;
-        b1e[al + PB * (b + PB * c)] = dot_row<PB, PBP>(SRy + b * PBP, v);
-      }
-    }
-    __syncthreads();
-    // ---- backward: S_x along alpha (line (b', c'), NC*NC lines per element), write out
-    if (tid < ne * NC * NC) {
-      const int le3 = tid / (NC * NC), q3 = tid - le3 * NC * NC;
-      const int b = C0 + q3 % NC, c = C0 + q3 / NC;
-      const T* SRx = SR(le3);
-      const T* b1e = B1(le3);
-      const int64_t e = e0 + le3;
-#pragma unroll
-      for (int al = 0; al < PB; ++al) v[al] = b1e[al + PB * (b + PB * c)];
-#pragma unroll OUT_UNR
-      for (int aa = 0; aa < NC; ++aa) {
-        const int a = C0 + aa;
-        const T acc = dot_row<PB, PBP>(SRx + a * PBP, v);
-        if constexpr (MODE == FDM_RAS) {
-          const int64_t li = e * (N * N * N) + (a - 1) + N * ((b - 1) + N * (c - 1));
-          const int mlog = __ffs(pflag[li] & 0x0F) - 1;   // 1/multiplicity: exact power of 2
-          const T wt = mlog == 0 ? T(1) : (mlog == 1 ? T(0.5) : (mlog == 2 ? T(0.25) : T(0.125)));
-          out[li] = io_cast<IO>(acc * wt);
-        } else {
-          out[e * PB3 + a + PB * (b + PB * c)] = io_cast<IO>(acc);
-        }
-      }
-    }
-  }
+// rbar = R_e r (se_pmg_gather_ext): one thread per window point.
+template <int P>
+__global__ void __launch_bounds__(256) fdm_gather_kernel(int64_t E, const int* __restrict__ nbr,
+                                                         const double* __restrict__ in,
+                                                         double* __restrict__ out) {
+  constexpr int PB = P + 3, PB3 = PB * PB * PB;
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= E * PB3) return;
+  const int64_t e = t / PB3;
+  const int q = (int)(t - e * PB3);
+  const int64_t src = window_source<P>(nbr + 27 * e, e, q % PB, (q / PB) % PB, q / (PB * PB));
+  out[t] = src >= 0 ? in[src] : 0.0;
 }
 
 // ------------------------------------------------------------------ FP32: one warp per element
@@ -1052,26 +834,15 @@ __global__ void __launch_bounds__(64, Fdm32PipeDims<P + 3>::BLOCKS_PER_SM)
   }
 }
 
-// Shared bytes per element: fdm_kernel<P, double, *> (two window buffers, S^T and S, the
-// eigenvalues, 27 neighbour ids) or fdm32_warp_kernel<P, *> (Fdm32Dims<P + 3>::PER floats, and
-// the block's window tables once per block).
-template <int P, typename T>
-constexpr size_t fdm_smem_per_element() {
-  if constexpr (sizeof(T) == 4) {
-    return Fdm32Dims<P + 3>::PER * sizeof(float);
-  } else {
-    using Dm = FdmDims<P + 3>;
-    return (2 * Dm::PB3P + 2 * Dm::SROW + (3 * (P + 3) + 3) / 4 * 4) * sizeof(T) + 27 * sizeof(int);
-  }
-}
-
+// Shared memory of a block: FP32 fdm32_warp_kernel (Fdm32Dims<P + 3>::PER floats per element, and the
+// block's window tables), FP64 fdm_fx_kernel.
 size_t fdm_smem_bytes(int p, bool fp32, int ne) {
   size_t per = 0, fixed = 0;  // per element; per block (the FP32 kernel's window tables)
   switch (p) {
 #define SE_FDM_SM(PP)                                   \
   case PP:                                              \
     if (fp32) {                                         \
-      per = fdm_smem_per_element<PP, float>();          \
+      per = Fdm32Dims<PP + 3>::PER * sizeof(float);     \
       fixed = Fdm32Dims<PP + 3>::TAB_BYTES;             \
     } else {                                            \
       per = fdm_fx_smem_per_element(PP);                \
@@ -1085,7 +856,7 @@ size_t fdm_smem_bytes(int p, bool fp32, int ne) {
   return per * ne + fixed;
 }
 
-// Largest block: 256 threads for fdm32_warp_kernel (its launch bounds), 512 in FP64 and df64.
+// Largest block: 256 threads for fdm32_warp_kernel (its launch bounds), 512 in FP64.
 int fdm_max_threads(bool fp32) { return fp32 ? 256 : 512; }
 
 // Threads of a block with ne elements: FP32 one warp per element, FP64 one per line of a phase.
@@ -1145,47 +916,10 @@ static int launch_fdm(const Level& lv, const T* in, const T* S, const T* lam, T*
     SE_CUDA(attr);
     fdm32_warp_kernel<P, MODE><<<blocks, threads, smem, s>>>(lv.E, lv.nbr, in, S, lam, lv.pflag, out);
   } else if constexpr (MODE == FDM_GATHER) {
-    static const cudaError_t attr = cudaFuncSetAttribute(
-        fdm_kernel<P, T, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    SE_CUDA(attr);
-    fdm_kernel<P, T, MODE><<<blocks, threads, fdm_smem_per_element<P, T>() * NE, s>>>(
-        lv.E, NE, lv.nbr, in, S, lam, lv.fdm_dinv64, lv.pflag, out);
+    fdm_gather_kernel<P><<<grid_for(lv.E * (P + 3) * (P + 3) * (P + 3), 256), 256, 0, s>>>(lv.E, lv.nbr, in, out);
   } else {
     return fdm_fx_apply(lv, MODE, in, out, NE, s);
   }
-  SE_LAUNCH_CHECK();
-  return SE_OK;
-}
-
-// df64 arithmetic on FP64 vectors: the FP64 kernel's layout (df64 values are 8 bytes, as FP64
-// ones), its S and Lambda from the df64 copies.  Fewer elements per block than FP64 (measured
-// on GB300 at 32^3 elements: p = 7 3 elements, 1.31 ms against 1.47 ms with FP64's 4; p = 5 3;
-// p = 3 6), unless a tile is set for FP64.
-static int fdm_df_elems_per_block(int p) {
-  if (tile_get(p, false).fdm_ne > 0) return fdm_elems_per_block(p, false);
-  switch (p) {
-    case 1: return 16;
-    case 2: return 10;
-    case 3: return 6;
-    case 4: return 5;
-    case 5: return 3;
-    case 6: return 3;
-    case 7: return 3;
-    default: return 2;
-  }
-}
-
-template <int P, int MODE>
-static int launch_fdm_df(const Level& lv, const double* in, double* out, cudaStream_t s) {
-  const int NE = fdm_df_elems_per_block(P);
-  const int threads = fdm_block_threads(P, false, NE);
-  const size_t smem = fdm_smem_per_element<P, double>() * NE;
-  const unsigned blocks = (unsigned)((lv.E + NE - 1) / NE);
-  static const cudaError_t attr = cudaFuncSetAttribute(
-      fdm_kernel<P, df64, MODE, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-  SE_CUDA(attr);
-  fdm_kernel<P, df64, MODE, double><<<blocks, threads, smem, s>>>(lv.E, NE, lv.nbr, in, lv.Sdf, lv.lamdf,
-                                                                   lv.fdm_dinv64, lv.pflag, out);
   SE_LAUNCH_CHECK();
   return SE_OK;
 }
@@ -1205,22 +939,8 @@ static int dispatch_fdm(const Level& lv, const T* in, T* out, cudaStream_t s) {
   const double PB = lv.p + 3.0, N = lv.N;
   const double fl = 2.0 * (3.0 * PB * PB * PB * PB + PB * PB * PB * N + PB * PB * N * N + PB * N * N * N) + PB * PB * PB;
   const double by = (PB * PB * PB + N * N * N + 3 * PB * PB + 3 * PB + (sizeof(T) == 8 ? PB * PB * PB : 0)) * sizeof(T);
-  bool use_df = false;
-  if constexpr (sizeof(T) == 8) use_df = MODE != FDM_GATHER && lv.df && lv.Sdf;
   ProfScope prof(SE_K_FDM, s, (double)lv.E, by * lv.E, fl * lv.E,
-                 use_df ? lv.p + 64 : prof_variant<T>(lv.p));
-  if constexpr (sizeof(T) == 8 && MODE != FDM_GATHER) {
-    if (use_df) {
-      switch (lv.p) {
-#define SE_FDM_DF(PP) \
-  case PP: return launch_fdm_df<PP, MODE>(lv, in, out, s);
-        SE_FDM_DF(1) SE_FDM_DF(2) SE_FDM_DF(3) SE_FDM_DF(4) SE_FDM_DF(5)
-        SE_FDM_DF(6) SE_FDM_DF(7) SE_FDM_DF(8) SE_FDM_DF(9) SE_FDM_DF(10)
-#undef SE_FDM_DF
-        default: break;
-      }
-    }
-  }
+                 prof_variant<T>(lv.p));
   switch (lv.p) {
 #define SE_FDM_CASE(PP) \
   case PP: return launch_fdm<PP, T, MODE>(lv, in, S, lam, out, s);

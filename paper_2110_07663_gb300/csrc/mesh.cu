@@ -222,13 +222,6 @@ int build_level(se_mesh_s* m, int p, Level* lvp, Allocs& allocs, cudaStream_t s)
   SE_TRY(h2d(lv.D32, D32h, N * N * sizeof(float), s));
   SE_TRY(h2d(dxi, lv.basis.xi, N * sizeof(double), s));
   SE_TRY(h2d(dw, lv.basis.w, N * sizeof(double), s));
-  if (ax_eo_supported(p)) {
-    const int H = N / 2;
-    double tab[4 * (SE_MAX_ORDER + 1) * (SE_MAX_ORDER + 1) / 4 + 4];
-    ax_eo_tables(lv.basis, tab);
-    SE_TRY(dmalloc(allocs, &lv.eo64, 4 * H * H));
-    SE_TRY(h2d(lv.eo64, tab, 4 * H * H * sizeof(double), s));
-  }
 
   // geometry
   double* dverts = nullptr;

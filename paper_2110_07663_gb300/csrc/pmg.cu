@@ -306,50 +306,6 @@ static int arnoldi_level(se_pmg_s* P, int l, cudaStream_t s, double* lam_out) {
 }
 
 // ------------------------------------------------------------------ set-up
-// df64 arithmetic for the Arnoldi rounds of an FP64 or FP32 preconditioner: df64 copies of the
-// smoothed levels' geometry and FDM factors live only while the bounds are estimated (copies
-// the mesh already holds for its outer operator are used as they are).
-static int df_transient(const double* src, df64** dst, int64_t n, cudaStream_t s,
-                        std::vector<void*>& keep) {
-  void* p = nullptr;
-  SE_TRY(dmalloc_transient(&p, (size_t)n * sizeof(df64), s));
-  keep.push_back(p);
-  *dst = static_cast<df64*>(p);
-  return split_df(src, *dst, n, s);
-}
-
-static int arnoldi_df_begin(se_pmg_s* P, cudaStream_t s, std::vector<void*>& keep) {
-  for (int l = 0; l + 1 < P->nlev; ++l) {
-    Level& lv = *P->lv[l];
-    const int H = lv.N / 2, PB = lv.p + 3;
-    const bool eo = ax_eo_supported(lv.p) && lv.eo64;
-    if (!lv.Gdf) SE_TRY(df_transient(lv.G64, &lv.Gdf, 6 * lv.L, s, keep));
-    if (eo && !lv.eodf) SE_TRY(df_transient(lv.eo64, &lv.eodf, 4 * H * H, s, keep));
-    if (!eo && !lv.Ddf) SE_TRY(df_transient(lv.D64, &lv.Ddf, (int64_t)lv.N * lv.N, s, keep));
-    if (lv.S64 && !lv.Sdf) {
-      SE_TRY(df_transient(lv.S64, &lv.Sdf, 3 * lv.E * PB * PB, s, keep));
-      SE_TRY(df_transient(lv.lam64, &lv.lamdf, 3 * lv.E * PB, s, keep));
-    }
-    lv.df = true;
-  }
-  return SE_OK;
-}
-
-static void arnoldi_df_end(se_pmg_s* P, cudaStream_t s, std::vector<void*>& keep) {
-  auto owned = [&](void* p) { return std::find(keep.begin(), keep.end(), p) != keep.end(); };
-  for (int l = 0; l + 1 < P->nlev; ++l) {
-    Level& lv = *P->lv[l];
-    lv.df = false;
-    if (owned(lv.Gdf)) lv.Gdf = nullptr;
-    if (owned(lv.eodf)) lv.eodf = nullptr;
-    if (owned(lv.Ddf)) lv.Ddf = nullptr;
-    if (owned(lv.Sdf)) lv.Sdf = nullptr;
-    if (owned(lv.lamdf)) lv.lamdf = nullptr;
-  }
-  for (void* p : keep) cudaFreeAsync(p, s);
-  keep.clear();
-}
-
 template <class T>
 static int alloc_vecs(se_pmg_s* P, int l) {
   LevelVecs<T>& V = P->vecs<T>(l);
@@ -367,10 +323,7 @@ static int pmg_build(se_pmg_s* P) {
   cudaStream_t s = P->stream;
   const se_pmg_desc& d = P->desc;
   const bool fp32 = d.precision == SE_FP32;
-  const bool df = d.precision == SE_DF64;
   SE_TRY(scratch_alloc(P->allocs, &P->scratch));
-  // df64 copies of the fine geometry belong to the mesh (the outer operator may use them too)
-  if (df) SE_TRY(make_df_geometry(m->fine, m->allocs, s));
   P->owned[0] = m->fine;  // shallow copy: shares the mesh's geometry and maps
   P->owned[0].G32 = nullptr;
   P->lv[0] = &P->owned[0];
@@ -383,12 +336,8 @@ static int pmg_build(se_pmg_s* P) {
     Level& lv = *P->lv[l];
     const bool coarsest = l == P->nlev - 1;
     if (fp32 && !coarsest) SE_TRY(make_fp32_geometry(lv, P->allocs, s));
-    if (df && !coarsest) {
-      SE_TRY(make_df_geometry(lv, P->allocs, s));
-      lv.df = true;
-    }
     if (!coarsest && d.smoother != SE_SMOOTH_JACOBI) {
-      SE_TRY(fdm_setup(m, lv, P->allocs, fp32, s, df));
+      SE_TRY(fdm_setup(m, lv, P->allocs, fp32, s));
       if (d.smoother == SE_SMOOTH_ASM) {
         const int64_t n3 = lv.E * (int64_t)(lv.p + 3) * (lv.p + 3) * (lv.p + 3);
         SE_TRY(dmalloc(P->allocs, &lv.ext64, n3));
@@ -414,15 +363,7 @@ static int pmg_build(se_pmg_s* P) {
     else SE_TRY(alloc_vecs<double>(P, l));
   }
   // the coarse level always solves in FP64 from the V-cycle's precision; Arnoldi needs FP64
-  // vectors (and FP64 or df64 arithmetic)
-  std::vector<void*> transient;
-  if (!df && d.arnoldi_df64) {
-    const int rb = arnoldi_df_begin(P, s, transient);
-    if (rb != SE_OK) {
-      arnoldi_df_end(P, s, transient);
-      return rb;
-    }
-  }
+  // vectors
   SE_CUDA(cudaStreamSynchronize(s));
   int rc = SE_OK;
   for (int l = 0; l + 1 < P->nlev && rc == SE_OK; ++l) {
@@ -432,7 +373,6 @@ static int pmg_build(se_pmg_s* P) {
     P->lmin[l] = d.eig_lo * lam;
     P->lmax[l] = d.eig_hi * lam;
   }
-  if (!df && d.arnoldi_df64) arnoldi_df_end(P, s, transient);
   SE_TRY(rc);
   SE_CUDA(cudaStreamSynchronize(s));
   return SE_OK;

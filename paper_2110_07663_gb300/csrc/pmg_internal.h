@@ -12,7 +12,7 @@ struct LevelVecs {
 
 int pmg_apply(se_pmg_s* P, const double* r, double* z, cudaStream_t s);
 int graph_solve_launch(se_mesh_s* m, se_pmg_s* P, const double* b, double* x, double tol,
-                       int maxit, cudaStream_t s, int tol_norm = SE_TOL_R0, int op_df = 0);
+                       int maxit, cudaStream_t s, int tol_norm = SE_TOL_R0);
 int graph_solve_result(se_mesh_s* m, cudaStream_t s, double tol, int maxit, se_solve_stats* st);
 // Pieces of the device-driven FPCG graph (solve.cu), shared with the batched solves (batch.cu).
 int prepare_graph_solve(se_mesh_s* m);
@@ -20,7 +20,7 @@ int read_graph_stats(se_mesh_s* m, cudaStream_t s, se_solve_stats* out, double t
 // Appends one whole FPCG solve of mesh m (x0 = the content of x at launch) to graph G as a branch
 // independent of the rest of G.
 int append_fpcg_solve(cudaGraph_t G, cudaStream_t cs, se_mesh_s* m, se_pmg_s* P, const double* b,
-                      double* x, double tol, int maxit, int tol_norm, int op_df);
+                      double* x, double tol, int maxit, int tol_norm);
 // Adds a conditional node at the capture frontier of cs and moves the frontier after it.
 int add_conditional(cudaStream_t cs, cudaGraphConditionalHandle h, cudaGraphConditionalNodeType type,
                     cudaGraph_t* body);

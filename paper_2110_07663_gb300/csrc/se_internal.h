@@ -9,7 +9,6 @@
 #include <vector>
 
 #include "se.h"
-#include "df64.h"
 
 namespace se {
 
@@ -115,15 +114,6 @@ struct Level {
   float* dinv32 = nullptr;
   uint8_t* pflag = nullptr;  // multiplicity and free bit [L]
   double* D64 = nullptr;     // derivative matrix on the device [N*N]
-  double* eo64 = nullptr;    // even-odd folded D and D^T tables [4][N/2][N/2] (even N)
-  // double-float copies for the operator and FDM kernels of SE_DF64 levels (FP64 vectors,
-  // df64 arithmetic); `df` routes those two kernels of this level to them
-  bool df = false;
-  df64* Gdf = nullptr;       // [6][L]
-  df64* eodf = nullptr;      // [4][N/2][N/2] (even N)
-  df64* Ddf = nullptr;       // [N][N] (odd N)
-  df64* Sdf = nullptr;       // [E][3][pb][pb]
-  df64* lamdf = nullptr;     // [E][3][pb]
   float* D32 = nullptr;
   const int* nbr = nullptr;  // element neighbours [E][27] (owned by the mesh)
   // fast diagonalisation factors (all levels but the coarsest)
@@ -204,7 +194,6 @@ struct se_mesh_s {
   double gtol = 0.0;
   int gmaxit = 0;
   int gtolnorm = 0;
-  int gopdf = 0;
 };
 
 namespace se {
@@ -229,8 +218,8 @@ template <class T>
 int gsmap_apply(const Level& lv, T* u, bool mask, cudaStream_t s);
 // Builds lv's index map from its lattice numbering (SE_MESH_GS_MAP).
 int build_level_gsmap(Level& lv, Allocs& allocs, cudaStream_t s);
-// FP64 operator with the x part of QQ^T and the mask inside the even-odd kernel (even N, box
-// lattice, sweeps): y = A u, or b - A u when b is given; the x-interfaces between the kernel's
+// FP64 operator with the x part of QQ^T and the mask inside the operator kernel (box lattice,
+// sweeps): y = A u, or b - A u when b is given; the x-interfaces between the kernel's
 // blocks, then the y/z launch follow (ax.cu).
 bool ax_fold_ok(const Level& lv);
 // dinv: y = A (dinv .* u) (the input scaled as it is loaded)
@@ -307,8 +296,7 @@ int fdm_apply_ext(const Level& lv, const T* rbar, T* zbar, cudaStream_t s);
 // elements per block.
 int fdm_fx_apply(const Level& lv, int mode, const double* in, double* out, int NE, cudaStream_t s);
 size_t fdm_fx_smem_per_element(int p);
-int fdm_setup(const se_mesh_s* m, Level& lv, Allocs& allocs, bool want32, cudaStream_t s,
-              bool want_df = false);
+int fdm_setup(const se_mesh_s* m, Level& lv, Allocs& allocs, bool want32, cudaStream_t s);
 int asm_weights(Level& lv, Allocs& allocs, cudaStream_t s);
 // Transfers (transfer.cu): level f (fine) <-> level c (coarse); FP64 by transfer_fx (block floating
 // point, transfer_fx.cu), which leaves out the restriction's QQ^T
@@ -364,8 +352,7 @@ int build_gsmap_from_gid(Level& lv, const int64_t* gid, const uint8_t* dirichlet
                          cudaStream_t s);
 
 // ------------------------------------------------------------------ profiling (common.cu)
-// Profiling variant of a launch: polynomial order p (0..31) plus 32 for FP32 arithmetic, plus 64
-// for double-float (df64) arithmetic on FP64 vectors.
+// Profiling variant of a launch: polynomial order p (0..31) plus 32 for FP32 arithmetic.
 constexpr int PROF_VARIANTS = 96;
 template <class T>
 inline int prof_variant(int p) {
@@ -401,20 +388,8 @@ int ax_local_tma(const Level& lv, const float* u, float* y, cudaStream_t s, cons
 // block) and the mask.
 int ax_local_fx(const Level& lv, const double* u, double* y, bool mask_in, const double* sub,
                 const double* dinv, int NE, bool fold, cudaStream_t s);
-// Even-odd folded df64 kernel (even N).
-bool ax_eo_supported(int p);
-void ax_eo_tables(const Basis1D& b, double* out);
 // The x-interfaces between consecutive blocks of ax_local_fx with fold (NE elements per block).
 int gs_fold_fixup(const Level& lv, double* y, int NE, cudaStream_t s);
-// The same contractions in df64 arithmetic (FP64 in and out); needs lv.Gdf and lv.eodf.
-int ax_local_eo_df(const Level& lv, const double* u, double* y, cudaStream_t s, const double* sub);
-// b[i] = nearest df64 of a[i] (device arrays, stream-ordered).
-int split_df(const double* a, df64* b, int64_t n, cudaStream_t s);
-// df64 copies of a level's geometric factors and folded tables (no-op if present).
-int make_df_geometry(Level& lv, Allocs& allocs, cudaStream_t s);
-inline bool ax_df_route(const Level& lv) {
-  return lv.df && lv.Gdf && (ax_eo_supported(lv.p) ? lv.eodf != nullptr : lv.Ddf != nullptr);
-}
 // SE_ETIMEOUT (and the record cleared) if a pipelined kernel of lv gave up a bounded wait since
 // the last call; synchronises s first.
 int level_pipeline_take(const Level& lv, cudaStream_t s);

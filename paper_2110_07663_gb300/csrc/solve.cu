@@ -42,18 +42,10 @@ static int read_scalars(se_mesh_s* m, cudaStream_t s, int count) {
   return SE_OK;
 }
 
-// The fine level as the outer operator sees it: FP64 arithmetic, or df64 (operator_df64) where
-// the mesh holds df64 geometry.
-static Level outer_level(const se_mesh_s* m, int op_df) {
-  Level lv = m->fine;
-  lv.df = op_df != 0;
-  return lv;
-}
-
 // Flexible PCG: beta = (z_{k+1}, r_{k+1} - r_k) / (z_k, r_k).
 static int fpcg(se_mesh_s* m, se_pmg_s* P, const double* b, double* x, const se_solve_opts& o,
                 cudaStream_t s, se_solve_stats* st) {
-  const Level lv = outer_level(m, o.operator_df64);
+  const Level& lv = m->fine;
   Scratch& sc = m->scratch;
   double *r = m->sr, *r2 = m->sr2, *z = m->sz, *p = m->sp, *w = m->sw;
   SE_TRY(ax_apply<double>(lv, x, w, s));
@@ -95,7 +87,7 @@ static int fpcg(se_mesh_s* m, se_pmg_s* P, const double* b, double* x, const se_
 // Givens rotations on the host; x += Z y at the end of each cycle.
 static int fgmres(se_mesh_s* m, se_pmg_s* P, const double* b, double* x, const se_solve_opts& o,
                   cudaStream_t s, se_solve_stats* st) {
-  const Level lv = outer_level(m, o.operator_df64);
+  const Level& lv = m->fine;
   const int64_t L = lv.L;
   Scratch& sc = m->scratch;
   const int mr = o.restart;
@@ -192,7 +184,6 @@ extern "C" int se_solve(se_mesh_t m, se_pmg_t P, const double* b, double* x,
   SE_CHECK(o.operator_df64 == 0 || o.operator_df64 == 1, SE_EINVAL, "se_solve: operator_df64");
   cudaStream_t s = as_stream(o.stream, m->stream);
   SE_TRY(ensure_solve_work(m, o.restart, o.method == SE_FGMRES));
-  if (o.operator_df64) SE_TRY(make_df_geometry(m->fine, m->allocs, s));
   se_solve_stats st{};
   SE_CUDA(cudaEventRecord(m->ev0, s));
   int rc;
@@ -287,9 +278,8 @@ int add_conditional(cudaStream_t cs, cudaGraphConditionalHandle h,
 // Appends one whole FPCG solve (x0 = the content of x at launch) to graph G, independent of the
 // rest of G.  All buffers must already exist: nothing is allocated while capturing.
 int append_fpcg_solve(cudaGraph_t G, cudaStream_t cs, se_mesh_s* m, se_pmg_s* P,
-                             const double* b, double* x, double tol, int maxit, int tol_norm,
-                             int op_df) {
-  const Level lv = outer_level(m, op_df);
+                             const double* b, double* x, double tol, int maxit, int tol_norm) {
+  const Level& lv = m->fine;
   Scratch& sc = m->scratch;
   double *r = m->sr, *r_old = m->sr2, *z = m->sz, *p = m->sp, *w = m->sw;
   DevStats* st = static_cast<DevStats*>(m->gstats);
@@ -369,12 +359,11 @@ int read_graph_stats(se_mesh_s* m, cudaStream_t s, se_solve_stats* out, double t
 // Builds (or reuses) this mesh's solve graph for (P, b, x, tol, maxit) and launches it on s
 // without waiting.  read_graph_stats collects the result.
 int graph_solve_launch(se_mesh_s* m, se_pmg_s* P, const double* b, double* x, double tol,
-                       int maxit, cudaStream_t s, int tol_norm, int op_df) {
+                       int maxit, cudaStream_t s, int tol_norm) {
   SE_TRY(prepare_graph_solve(m));
   const uint64_t uid = P ? P->uid : 0;
   const bool same = m->gexec && m->gkey[0] == P && m->gpmg_uid == uid && m->gkey[1] == b && m->gkey[2] == x &&
-                    m->gtol == tol && m->gmaxit == maxit && m->gtolnorm == tol_norm &&
-                    m->gopdf == op_df;
+                    m->gtol == tol && m->gmaxit == maxit && m->gtolnorm == tol_norm;
   if (!same) {
     if (m->gexec) cudaGraphExecDestroy(m->gexec);
     m->gexec = nullptr;
@@ -382,7 +371,7 @@ int graph_solve_launch(se_mesh_s* m, se_pmg_s* P, const double* b, double* x, do
     SE_CUDA(cudaGraphCreate(&G, 0));
     cudaStream_t cs;
     SE_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
-    int rc = append_fpcg_solve(G, cs, m, P, b, x, tol, maxit, tol_norm, op_df);
+    int rc = append_fpcg_solve(G, cs, m, P, b, x, tol, maxit, tol_norm);
     cudaStreamDestroy(cs);
     if (rc == SE_OK) {
       cudaError_t e = cudaGraphInstantiate(&m->gexec, G, 0);
@@ -401,7 +390,6 @@ int graph_solve_launch(se_mesh_s* m, se_pmg_s* P, const double* b, double* x, do
     m->gtol = tol;
     m->gmaxit = maxit;
     m->gtolnorm = tol_norm;
-    m->gopdf = op_df;
   }
   SE_CUDA(cudaGraphLaunch(m->gexec, s));
   return SE_OK;
@@ -414,7 +402,7 @@ int graph_solve_result(se_mesh_s* m, cudaStream_t s, double tol, int maxit, se_s
 // se_solve with graph_capture: one launch of the cached graph, then its statistics.
 int graph_solve(se_mesh_s* m, se_pmg_s* P, const double* b, double* x, const se_solve_opts& o,
                 cudaStream_t s, se_solve_stats* st) {
-  SE_TRY(graph_solve_launch(m, P, b, x, o.tol, o.maxit, s, o.tol_norm, o.operator_df64));
+  SE_TRY(graph_solve_launch(m, P, b, x, o.tol, o.maxit, s, o.tol_norm));
   return read_graph_stats(m, s, st, o.tol, o.maxit);
 }
 
