@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(512) ax_local_kernel(int64_t E, int NE, const 
 
 // Elements per block for N*N threads per element: the tuned value if one is set and valid,
 // else enough elements for about 256 threads.
-int ax_elems_per_block(int p, bool fp32) {
+int ax_elems_per_block(int p, bool fp32, int64_t E) {
   const int N = p + 1;
   const int t = tile_get(p, fp32).ax_ne;
   if (t >= 1 && t * N * N <= 512) return t;
@@ -114,7 +114,7 @@ int ax_elems_per_block(int p, bool fp32) {
   // and several small blocks per SM, which hide each other's barriers
   if (!fp32) {
     constexpr int ne64[SE_MAX_ORDER + 2] = {0, 0, 32, 14, 4, 10, 7, 5, 2, 3, 2, 1};
-    return ne64[N];
+    return balanced_elems(E, ne64[N]);
   }
   const int ne = 256 / (N * N);
   return ne < 1 ? 1 : ne;
@@ -150,7 +150,7 @@ int ax_local(const Level& lv, const T* u, T* y, bool mask_in, cudaStream_t s, co
   if constexpr (sizeof(T) == 4) {
     if (!mask_in && ax_tma_supported(lv.p)) return ax_local_tma(lv, u, y, s, sub);
   } else {
-    return ax_local_fx(lv, u, y, mask_in, sub, nullptr, ax_elems_per_block(lv.p, false), false, s);
+    return ax_local_fx(lv, u, y, mask_in, sub, nullptr, ax_elems_per_block(lv.p, false, lv.E), false, s);
   }
   if constexpr (sizeof(T) == 4) {
     switch (N) {
@@ -601,7 +601,7 @@ static int gs_after_fold(const Level& lv, double* y, int NE, cudaStream_t s) {
 
 int ax_apply_folded(const Level& lv, const double* u, double* y, const double* b, cudaStream_t s,
                     const double* dinv, bool mask_in) {
-  const int NE = ax_elems_per_block(lv.p, false);
+  const int NE = ax_elems_per_block(lv.p, false, lv.E);
   {
     const double pts = (double)lv.L;
     // u, y, 6 geometric factors, b (residual form) and D^-1 (scaled input) per point; the

@@ -867,7 +867,7 @@ int fdm_block_threads(int p, bool fp32, int ne) {
 
 // Elements per block: the tuned value if one is set and valid; else FP32 8 (one warp each),
 // FP64 about 300 lines per phase (at most 16 elements).
-int fdm_elems_per_block(int p, bool fp32) {
+int fdm_elems_per_block(int p, bool fp32, int64_t E) {
   const int PB = p + 3;
   const int t = tile_get(p, fp32).fdm_ne;
   if (t >= 1 && t <= 16 && fdm_block_threads(p, fp32, t) <= fdm_max_threads(fp32) &&
@@ -878,7 +878,7 @@ int fdm_elems_per_block(int p, bool fp32) {
   // p = 7, 24^3: 1 485, 2 424, 3 403, 4 442, 5 409; p = 8, 16^3: 1 193, 2 189, 3 181; p = 9, 16^3:
   // 1 282, 2 263, 3 255; p = 10, 14^3: 1 256, 2 269, 3 250.  Blocks of about 300 lines
   static const int ne64[SE_MAX_ORDER + 1] = {1, 16, 10, 7, 5, 4, 3, 3, 3, 3, 3};
-  int ne = fp32 ? 8 : ne64[p];
+  int ne = fp32 ? 8 : balanced_elems(E, ne64[p]);
   while (ne > 1 && fdm_smem_bytes(p, fp32, ne) > 200 * 1024) --ne;
   return ne;
 }
@@ -886,7 +886,7 @@ int fdm_elems_per_block(int p, bool fp32) {
 template <int P, typename T, int MODE>
 static int launch_fdm(const Level& lv, const T* in, const T* S, const T* lam, T* out,
                       cudaStream_t s) {
-  const int NE = fdm_elems_per_block(P, sizeof(T) == 4);
+  const int NE = fdm_elems_per_block(P, sizeof(T) == 4, lv.E);
   const int threads = fdm_block_threads(P, sizeof(T) == 4, NE);
   const size_t smem = fdm_smem_bytes(P, sizeof(T) == 4, NE);
   const unsigned blocks = (unsigned)((lv.E + NE - 1) / NE);

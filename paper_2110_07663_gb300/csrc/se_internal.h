@@ -378,7 +378,10 @@ struct TileCfg {
 };
 TileCfg tile_get(int p, bool fp32);
 void tile_set(int p, bool fp32, const TileCfg& c);
-int ax_elems_per_block(int p, bool fp32);
+int ax_elems_per_block(int p, bool fp32, int64_t E = 0);  // E: the level's elements, 0 for many
+// At most `most` elements per block of the FP64 operator and FDM kernels, fewer where the E elements
+// would leave multiprocessors idle or unevenly loaded.
+int balanced_elems(int64_t E, int most);
 // FP32 Ax pipelined with TMA bulk copies (even N only); device status of its bounded waits.
 bool ax_tma_supported(int p);
 int ax_tma_group(int p);
@@ -393,7 +396,7 @@ int gs_fold_fixup(const Level& lv, double* y, int NE, cudaStream_t s);
 // SE_ETIMEOUT (and the record cleared) if a pipelined kernel of lv gave up a bounded wait since
 // the last call; synchronises s first.
 int level_pipeline_take(const Level& lv, cudaStream_t s);
-int fdm_elems_per_block(int p, bool fp32);
+int fdm_elems_per_block(int p, bool fp32, int64_t E = 0);
 size_t fdm_smem_bytes(int p, bool fp32, int ne);
 int fdm_block_threads(int p, bool fp32, int ne);
 int fdm_max_threads(bool fp32);
