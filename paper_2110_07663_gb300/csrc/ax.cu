@@ -401,8 +401,11 @@ __global__ void gs_mask_faces(int nx, int ny, int nz, int bits, T* __restrict__ 
 // 24^3 52 / 59, 32^3 114 / 133; p = 3, 16^3 (0.26M) 9.6 / 7.0, 24^3 (0.9M) 13.2 / 13.6, 32^3 19.4 / 22.6;
 // p = 1, 32^3 (0.26M) 12.6 / 8.5.  After the folded operator (fix-up and y/z launch against one): p = 7,
 // 4^3 23.0 / 19.8 with the operator, 12^3 41.3 / 38.9; p = 3, 24^3 36.4 / 39.0.
-constexpr int64_t GS_ONE_LAUNCH_POINTS = 600000;
-static bool gs_one_launch(const Level& lv) { return lv.L <= GS_ONE_LAUNCH_POINTS; }
+// In solves the launches are closer together: FP64 14^3 p = 7 (1.4M) 12.44 ms either way, 20^3 (4.1M)
+// 17.55 / 18.15.  FP32 (half the bytes; us of the FP32 operator): 12^3 p = 9 (1.7M) 52.8 / 48.9, 20^3 p = 7
+// (4.1M) 101.3 / 95.7; solve 14^3 p = 7 5.72 / 5.41 ms.
+template <typename T>
+static bool gs_one_launch(const Level& lv) { return lv.L <= (sizeof(T) == 4 ? 5000000 : 1300000); }
 
 // QQ^T in one launch: a thread per point on an element's upper faces (i, j or k = p) whose copies the
 // element owns (no lower neighbour shares them) gathers the node's 2, 4 or 8 copies, sums them in the
@@ -525,7 +528,7 @@ static int gs_sweeps(const Level& lv, T* u, bool mask, double bytes, double flop
   if (mask)
     for (int f = 0; f < 6; ++f)
       if (lv.bc[f] == SE_BC_DIRICHLET) bits |= 1 << f;
-  if (gs_one_launch(lv)) return gs_all<T, N>(lv, 0, bits, u, var, bytes, flops, s);
+  if (gs_one_launch<T>(lv)) return gs_all<T, N>(lv, 0, bits, u, var, bytes, flops, s);
   if (bits && nx == 1) {  // no x sweep to carry the mask
     {
       const int64_t n = 2 * N2 * ((int64_t)ny * nz + (int64_t)nx * nz + (int64_t)nx * ny);
@@ -586,7 +589,7 @@ static int gs_after_fold(const Level& lv, double* y, int NE, cudaStream_t s) {
   // the x direction must be complete before the y sweep adds across y-interfaces: a copy summed
   // across a block-boundary x-interface after the y sweep would count its y-partner's x-neighbour
   // twice
-  if (gs_one_launch(lv)) {
+  if (gs_one_launch<double>(lv)) {
     const double copies = yz_copies<N>(nx, ny, nz);
     return gs_all<double, N>(lv, NE, 0, y, var, 2.0 * copies * sizeof(double), copies / 2, s);
   }

@@ -157,7 +157,7 @@ def test_transfers_range_and_unscalable_values(pf, pc):
 
 
 @pytest.mark.parametrize("nel,p", [((1, 1, 1), 3), ((1, 4, 3), 2), ((5, 1, 2), 7), ((7, 6, 1), 4), ((9, 5, 4), 1),
-                                   ((30, 29, 31), 2), ((11, 12, 11), 7)])
+                                   ((30, 29, 31), 2), ((11, 12, 11), 7), ((16, 15, 14), 7)])
 @pytest.mark.parametrize("bc", [("D",) * 6, ("N", "D", "D", "N", "N", "N")])
 def test_qqt_one_launch_and_sweeps(nel, p, bc):
     """QQ^T with and without the mask on lattices one element wide in each direction, and on both sides
