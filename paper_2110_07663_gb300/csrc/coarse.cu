@@ -754,9 +754,12 @@ int coarse_alloc(const Level& lv, Allocs& allocs, CoarseWork* w) {
   }
   SE_CHECK(per_sm >= 1, SE_ECUDA, "coarse solver kernel cannot be resident");
   // one point per thread where possible; a grid of more than half the SMs is rounded up to a
-  // multiple of the SM count so that the FP64 work spreads evenly
+  // multiple of the SM count so that the FP64 work spreads evenly; fewer nodes: 128 per block while
+  // that leaves an SM for each (us per iteration with 256 / 128 / 64 / 32 nodes per block: n = 729
+  // 7.6 / 6.9 / 6.8 / 7.4, n = 4913 7.7 / 6.9 / 6.9 / 7.1, n = 15625 8.1 / 6.9 / 7.8 / 7.8)
   int64_t want = (n + CG_THREADS - 1) / CG_THREADS;
   if (want > sms / 2) want = (want + sms - 1) / sms * sms;
+  else want = std::min<int64_t>(sms, (n + CG_THREADS / 2 - 1) / (CG_THREADS / 2));
   const int64_t cap = (int64_t)sms * (per_sm < 2 ? per_sm : 2);
   if (want > cap) want = cap;
   if (want < 1) want = 1;
@@ -764,12 +767,11 @@ int coarse_alloc(const Level& lv, Allocs& allocs, CoarseWork* w) {
   for (double** v : {&w->x, &w->r, &w->u, &w->p, &w->q, &w->s, &w->z, &w->w0, &w->w1})
     SE_TRY(dmalloc(allocs, v, n));
   SE_TRY(dmalloc(allocs, &w->partial, coarse_partial_doubles(w->nblocks)));
-  SE_TRY(dmalloc(allocs, &w->bar, 2));
-  SE_TRY(dmalloc(allocs, &w->status, 2));
-  SE_TRY(dzero(w->bar, 2 * sizeof(unsigned), allocs.stream));
-  SE_TRY(dzero(w->status, 2 * sizeof(int), allocs.stream));
-  SE_TRY(dmalloc(allocs, &w->flags, (size_t)w->nblocks));
-  SE_TRY(dzero(w->flags, (size_t)w->nblocks * sizeof(unsigned), allocs.stream));
+  // count, status and flags in one piece: one reset per solve
+  SE_TRY(dmalloc(allocs, &w->bar, 4 + (size_t)w->nblocks));
+  w->status = reinterpret_cast<int*>(w->bar + 2);
+  w->flags = w->bar + 4;
+  SE_TRY(dzero(w->bar, (4 + (size_t)w->nblocks) * sizeof(unsigned), allocs.stream));
   SE_TRY(dmalloc(allocs, &w->totals, 3));
   SE_TRY(dzero(w->totals, 3 * sizeof(unsigned long long), allocs.stream));
   return SE_OK;
@@ -808,10 +810,9 @@ int coarse_solve(const Level& lv, CoarseWork& w, const T* r_l, T* x_l, double to
   a.maxit = maxit;
   a.timeout_ns = BARRIER_TIMEOUT_NS;
   ProfScope prof(SE_K_COARSE, s, (double)lv.n_global, 0.0, 0.0);
-  SE_CUDA(cudaMemsetAsync(w.bar, 0, 2 * sizeof(unsigned), s));
-  SE_CUDA(cudaMemsetAsync(w.status, 0, 2 * sizeof(int), s));
   const bool reg = w.flags && lv.n_global <= (int64_t)w.nblocks * CG_THREADS;
-  if (reg) SE_CUDA(cudaMemsetAsync(w.flags, 0, (size_t)w.nblocks * sizeof(unsigned), s));
+  // bar[2], status[2] and the flags are contiguous (coarse_alloc, the static work space)
+  SE_CUDA(cudaMemsetAsync(w.bar, 0, (4 + (reg ? (size_t)w.nblocks : 0)) * sizeof(unsigned), s));
   void* args[] = {&a};
   SE_TRY(coarse_kernel_attrs());
   SE_CUDA(cudaLaunchCooperativeKernel(reg ? (const void*)coarse_reg_kernel<T> : (const void*)coarse_pcg_kernel<T>,
