@@ -242,16 +242,19 @@ static int launch_ax_tma(const Level& lv, const float* u, float* y, int NE, cons
              : launch_ax_tma_t<N, false>(lv, u, y, NE, sub, s);
 }
 
-// Elements per group of the pipelined kernel (tuned value, else 2 groups of N^2 threads).
+// Elements per group of the pipelined kernel: the tuned value if one is set and valid, else about 128
+// threads.  Two stages of a group fill most of an SM's shared memory with 256 threads at p = 7 and 9, so
+// that one block and its barriers were alone on the SM; smaller groups leave room for 2 to 6 blocks,
+// whose loads and contractions overlap.  Measured on GB300 (us per launch by elements per group): p = 3,
+// 32^3: 4 18.5, 8 17.4, 16 18.5; p = 5, 32^3: 2 51.0, 3 49.2, 4 47.4, 7 49.1; p = 7, 12^3: 1 11.4, 2 11.4,
+// 4 12.3, 32^3: 1 90.7, 2 90.6, 3 91.7, 4 104.4 (5.9 TB/s of 8 values a point, 5.1 before); p = 9, 16^3:
+// 1 42.0, 2 51.2 (there shared-memory reads bound it).
 int ax_tma_group(int p) {
   const int N = p + 1;
   const int t = tile_get(p, true).ax_ne;
   // shared memory for the residual form (18 blocks of the group): the plain form (16) then fits too
   if (t >= 1 && t * N * N <= 512 && 18 * t * N * N * N * 4 <= 200 * 1024) return t;
-  int ne = 256 / (N * N);
-  if (ne < 1) ne = 1;
-  while (ne > 1 && 18 * ne * N * N * N * 4 > 200 * 1024) --ne;
-  return ne;
+  return N <= 2 ? 32 : (N <= 4 ? 8 : (N <= 6 ? 4 : (N <= 8 ? 2 : 1)));
 }
 
 bool ax_tma_supported(int p) { return (p + 1) % 2 == 0 && p + 1 >= 2 && p + 1 <= 10; }

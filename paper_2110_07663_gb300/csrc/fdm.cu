@@ -865,8 +865,8 @@ int fdm_block_threads(int p, bool fp32, int ne) {
   return fp32 ? 32 * ne : (ne * PB * PB + 31) / 32 * 32;
 }
 
-// Elements per block: the tuned value if one is set and valid; else FP32 8 (one warp each),
-// FP64 about 300 lines per phase (at most 16 elements).
+// Elements per block: the tuned value if one is set and valid; else FP32 8 or, on small levels, 4 (one
+// warp each), FP64 about 300 lines per phase (at most 16 elements).
 int fdm_elems_per_block(int p, bool fp32, int64_t E) {
   const int PB = p + 3;
   const int t = tile_get(p, fp32).fdm_ne;
@@ -878,7 +878,13 @@ int fdm_elems_per_block(int p, bool fp32, int64_t E) {
   // p = 7, 24^3: 1 485, 2 424, 3 403, 4 442, 5 409; p = 8, 16^3: 1 193, 2 189, 3 181; p = 9, 16^3:
   // 1 282, 2 263, 3 255; p = 10, 14^3: 1 256, 2 269, 3 250.  Blocks of about 300 lines
   static const int ne64[SE_MAX_ORDER + 1] = {1, 16, 10, 7, 5, 4, 3, 3, 3, 3, 3};
-  int ne = fp32 ? 8 : balanced_elems(E, ne64[p]);
+  // FP32 (fdm32_warp_kernel; us by elements per block, 4 / 8): blocks of 4 spread a small level's warps
+  // over more SMs and leave less of the chip idle in the last wave; blocks of 8 share their window table
+  // among more elements.  RAS p = 9, 5^3 16.4 / 20.3, 12^3 26.2 / 29.4, 16^3 49.0 / 51.5, 18^3 65.8 / 64.0;
+  // p = 8, 12^3 22.2 / 24.7, 18^3 49.6 / 47.9; p = 6, 12^3 14.6 / 16.4, 20^3 39.2 / 37.7; p = 10, 4^3
+  // 20.8 / 24.8, 9^3 26.5 / 25.2, 13^3 45.0 / 37.3; ASM p = 7, 4^3 14.2 / 16.4, 12^3 20.4 / 22.7
+  const int ne32 = E > 0 && E <= (p < 10 ? 5000 : 600) ? 4 : 8;
+  int ne = fp32 ? ne32 : balanced_elems(E, ne64[p]);
   while (ne > 1 && fdm_smem_bytes(p, fp32, ne) > 200 * 1024) --ne;
   return ne;
 }
