@@ -24,8 +24,10 @@
 // Measured on GB300 (us per launch; in brackets the even-odd FP64 kernel this one replaced, which ran at
 // the FP64 pipe's 2 FMA/clk/SM): 32^3 elements p = 7 406 [1420], p = 5 198 [525], p = 3 54 [138]; even
 // orders (unfolded in FP64) 20^3 p = 8 182 [725].  Memory needs 158 us of the 406 and the 9 FP64
-// instructions per point 240; without both the kernel still takes 332: what bounds it is the issue of
-// about 430 instructions per 32 points, 72 of them multiply-adds of 3.5 cycles each.  64 registers beat
+// instructions per point 240; without both the kernel still takes 332: what bounds it is about 495
+// instructions per 32 points, 72 of them multiply-adds of 3.5 cycles each, at the 32 warps that its
+// registers and shared memory allow (busy: FP64 pipe 67%, multiply-adds 46%, other integer 44%, issue
+// 51%; none is full, each waits for the others in turn).  64 registers beat
 // 48, 56, 72 and more; prefetching G to L2 costs more instructions than it saves waits.  u on the
 // element's scale instead of each line's was 4% faster, but lost accuracy where values within an
 // element span many decades.
