@@ -16,6 +16,7 @@
 #include <mutex>
 #include <vector>
 
+#include "coarse_flags.h"
 #include "pmg_internal.h"
 
 namespace se {
@@ -530,13 +531,13 @@ __device__ bool grid_wait3(unsigned* count, unsigned call, int* status, unsigned
   return *(volatile int*)status == 0;
 }
 
-// Waits (bounded) until flags[b] >= want for every block b in [b0, b1]; warp 0 polls.
+// Waits (bounded) until every block b in [b0, b1] has published generation `want`; warp 0 polls.
 __device__ bool wait_flags(const unsigned* flags, int b0, int b1, unsigned want, int* status,
                            long long timeout_ns) {
   if (threadIdx.x < 32) {
     const long long t0 = global_ns();
     for (int b = b0 + (int)threadIdx.x; b <= b1; b += 32) {
-      while ((int)(load_acquire(flags + b) - want) < 0) {
+      while (!coarse_flag_reached(load_acquire(flags + b), want)) {
         if (*(volatile int*)status != 0) break;
         if (global_ns() - t0 > timeout_ns) {
           atomicExch(status, SE_ETIMEOUT);
@@ -589,14 +590,14 @@ __device__ __forceinline__ void coarse_pcg_reg(const CoarseArgs<T>& c, unsigned 
   }
   double v[3] = {r * u, w * u, r * r};
   unsigned call = 0;
-  grid_post3(c.count, call, nb, c.part, v, red, blk, myflag, 1u);
+  grid_post3(c.count, call, nb, c.part, v, red, blk, myflag, coarse_flag(0));
   int it = 0;
   double gamma = 0.0, alpha = 0.0, tol2 = 0.0;
   double R = 0.0, K = 0.0;  // thread 0: 1 / gamma_prev, 1 / (gamma_prev alpha_prev)
   bool ok = true;
   for (;;) {
-    // m = D^-1 w, n = Ahat w on this iteration's w (neighbours: generation it + 1 published)
-    ok = wait_flags(c.flags, b0, b1, (unsigned)(it + 1), c.status, c.timeout_ns);
+    // m = D^-1 w, n = Ahat w on this iteration's w (the neighbours have published it)
+    ok = wait_flags(c.flags, b0, b1, coarse_flag(it), c.status, c.timeout_ns);
     if (!ok) break;
     const double* wr = (it & 1) ? c.w1 : c.w0;
     double m = 0.0, nv = 0.0;
@@ -651,13 +652,13 @@ __device__ __forceinline__ void coarse_pcg_reg(const CoarseArgs<T>& c, unsigned 
     v[1] = w * u;
     v[2] = r * r;
     ++it;
-    grid_post3(c.count, call, nb, c.part, v, red, blk, myflag, (unsigned)(it + 1));
+    grid_post3(c.count, call, nb, c.part, v, red, blk, myflag, coarse_flag(it));
   }
   // x to memory, one more summing barrier (nothing summed), then each local copy takes its node
   if (ok) {
     if (act) c.x[g] = x;
     double zero[3] = {0.0, 0.0, 0.0}, unused;
-    grid_post3(c.count, call, nb, c.part, zero, red, blk, myflag, 0xffffffffu);
+    grid_post3(c.count, call, nb, c.part, zero, red, blk, myflag, coarse_flag_final(it));
     ok = grid_wait3(c.count, call++, c.status, nb, c.timeout_ns, c.part, zero, unused, red,
                     [](double (&)[3]) { return 0.0; });
   }
