@@ -238,7 +238,7 @@ __global__ void __maxnreg__(fdm_fx_regs<P>()) fdm_fx_kernel(const __grid_constan
         bad |= fx_bad(ms);
         int h, l;
         fx_split(s3[d], fx_exponent(ms), h, l);
-        const int up = l >> (FX_LIMB - 1);  // low limb of both signs (a bias in the dropped products otherwise)
+        const int up = (l + (int)FX_HALF) >> FX_LIMB;  // |low limb| <= 2^27 (larger dropped products otherwise)
         h += up;
         l -= up << FX_LIMB;
         SR[d * Dm::SMAT + lq * PBP + lp] = make_int2(h, l);

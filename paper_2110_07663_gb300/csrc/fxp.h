@@ -6,8 +6,9 @@
 // fixed point: three integer multiply-adds per term instead of one DFMA, 7 times the rate.
 //
 //   value      x = v 2^(56 - e), |x| < 2^57, e the (unbiased) exponent of the largest |v| of the
-//              line or element: kept as x = h 2^28 + l, h signed, 0 <= l <= 2^28 (fx_split; bits below
-//              2^-56 of the largest value are dropped)
+//              line or element: kept as x = h 2^28 + l, |l| < 2^28, h and l of the sign of v
+//              (fx_split; bits below 2^-56 of the largest value are dropped, and what is
+//              dropped whole contracts to exactly 0)
 //   matrix     M' = M 2^k rounded to an integer, |M'| < 2^59, kept as mh 2^28 + ml with
 //              -2^27 <= ml < 2^27 (fx_limbs), its row sums bounded so that the sums below fit
 //   product    hi = sum mh h, mid = sum (mh l + ml h), 64-bit sums that cannot overflow
@@ -193,9 +194,9 @@ SE_FX void fx_split(double v, int E, int& h, int& l) {
   const unsigned one = 1u << (20 + UP);
   const unsigned top = (fx_funnel_l(lo, hi, UP) & (one - 1u)) | one;
   const unsigned long long x = fx_shr(((unsigned long long)top << 32) | (lo << UP), sh);
-  const unsigned xl = (unsigned)x >> 4;
-  h = (int)(unsigned)(x >> 32) ^ s;
-  l = (int)((xl ^ (unsigned)s) & 0x0fffffffu) - s;
+  // both limbs take the sign: a zero, or a value shifted out, has two zero limbs whatever its sign
+  h = ((int)(unsigned)(x >> 32) ^ s) - s;
+  l = ((int)((unsigned)x >> 4) ^ s) - s;
 }
 
 // The double nearest to R 2^(eb - 1023), |R| < 2^63; eb >= 1 and eb + 63 < 2046 (callers bound
