@@ -1,18 +1,19 @@
 // FP64 local Ax with folded line contractions in block floating point (fxp.h), every N.
 //
 // Sum factorisation: (ur, us, ut) = (D_r u, D_s u, D_t u);  w = G (ur, us, ut);
-// y = D_r^T wr + D_s^T ws + D_t^T wt.  The six contractions run on the integer pipe: a line of u is
-// split into fixed point on the scale of its largest value (so that a result's error is relative to
-// its own line, as in FP64), the gradients come back as doubles for the pointwise product with G
-// (9 FP64 instructions per point, what is left on the FP64 pipe), w is split on the scale of the
-// element's largest value, and the three parts of y are added as 64-bit integers before the one
-// rounding to double.  The derivative matrix is centro-antisymmetric, so
-// a line of N values costs N^2/2 terms.
+// y = D_r^T wr + D_s^T ws + D_t^T wt.  The six contractions run on the integer pipe: every line, of u
+// and of w, is split into fixed point on the scale of its own largest value, so that a result's error is
+// relative to its lines, as in FP64.  The gradients come back as doubles for the pointwise product
+// with G (9 FP64 instructions per point, what is left on the FP64 pipe); the three parts of y stay
+// 64-bit integers with the scale of their line, are added on the largest of the three scales and
+// rounded to double once.  The derivative matrix is centro-antisymmetric, so a line of N values costs
+// N^2/2 terms.
 //
 // NE elements per block, N^2 threads per element; each thread owns one line per direction.  Per
 // element three arrays U, R, S in shared memory (rows of N padded to an odd stride, so that lines
-// along every direction are read without bank conflicts), each updated in place: a thread
-// writes a line's results over the line, and the column (i, j, 0..N-1) it owns holds wt in U.
+// along every direction are read without bank conflicts; the padding holds the lines' scales), each
+// updated in place: a thread writes a line's results over the line, and the column (i, j, 0..N-1)
+// it owns holds wt in U.
 //
 // FOLD: the block's elements are consecutive in the element numbering, so neighbours along x
 // (same row of the lattice, nx elements per row) are usually in the same block.  The kernel then
@@ -22,22 +23,24 @@
 // left to gs_fold_fixup_x.
 //
 // Measured on GB300 (us per launch; in brackets the even-odd FP64 kernel this one replaced, which ran at
-// the FP64 pipe's 2 FMA/clk/SM): 32^3 elements p = 7 406 [1420], p = 5 198 [525], p = 3 54 [138]; even
-// orders (unfolded in FP64) 20^3 p = 8 182 [725].  Memory needs 158 us of the 406 and the 9 FP64
-// instructions per point 240; without both the kernel still takes 332: what bounds it is about 495
-// instructions per 32 points, 72 of them multiply-adds of 3.5 cycles each, at the 32 warps that its
-// registers and shared memory allow (busy: FP64 pipe 67%, multiply-adds 46%, other integer 44%, issue
-// 51%; none is full, each waits for the others in turn).  64 registers beat
-// 48, 56, 72 and more; prefetching G to L2 costs more instructions than it saves waits.  u on the
-// element's scale instead of each line's was 4% faster, but lost accuracy where values within an
-// element span many decades.
+// the FP64 pipe's 2 FMA/clk/SM): 32^3 elements p = 7 420 [1420], p = 5 205 [525], p = 3 55 [138]; even
+// orders (unfolded in FP64) 20^3 p = 8 178 [725].  Memory needs 158 us of the 420 and the 9 FP64
+// instructions per point 240; what bounds it is about 500 instructions per 32 points, 72 of them
+// multiply-adds of 3.5 cycles each, at the 32 warps that its registers and shared memory allow (no
+// pipe is full, each waits for the others in turn).  64 registers beat 48, 56, 72 and more;
+// prefetching G to L2 costs more instructions than it saves waits.  w on one scale per element was 2%
+// faster at p = 7 (406), but a small value then lost the bits below 2^-56 of the element's largest one,
+// though no line joins them; the parts of y as doubles, added in FP64, cost about 470.
 //
-// Error against extended precision (2-norm, on this repository's meshes), over that of the FP64 dot
-// products: 0.6 to 0.75 for random values, 0.3 to 0.8 for smooth ones, 0.6 for values that decay by
-// eight decades across the element.
+// Error against extended precision (2-norm, host emulation on perturbed meshes, p = 2 to 10), over that
+// of the FP64 dot products: 0.37 to 0.78 for random values, 0.39 to 0.50 for smooth ones, 0.31 to
+// 0.56 for values that decay by eight decades across the element, 0.29 to 0.74 around one value 10^8
+// times the others; away from that value's lines the points keep FP64's accuracy.
 //
-// Elements whose values cannot share a scale (infinities, NaN, magnitudes at the ends of the
-// range) send their block to ax_slow_block, the same operator in FP64.
+// A line whose values cannot share a scale (infinities, NaN, magnitudes at the ends of the range) is
+// contracted in FP64 (ax_slow_line); what does not touch it keeps its bits.
+#include <climits>
+
 #include "fxp.h"
 #include "se_internal.h"
 
@@ -53,9 +56,10 @@ struct AxFxArgs {
   int nx, ny, nz, bits;    // FOLD
 };
 
-// Splits the line p[0], p[st], ... on its own scale and calls f(E); whether it could not.
-template <int N, class F>
-__device__ __forceinline__ bool fx_split_line(const double* p, int st, int (&h)[N], int (&l)[N], F&& f) {
+// Splits the line p[0], p[st], ... on its own scale E; false where it has none (infinities, NaN,
+// largest value at an end of the range).
+template <int N>
+__device__ __forceinline__ bool fx_split_line(const double* p, int st, int (&h)[N], int (&l)[N], int& E) {
   double v[N];
   unsigned mag = 0u;
 #pragma unroll
@@ -63,18 +67,50 @@ __device__ __forceinline__ bool fx_split_line(const double* p, int st, int (&h)[
     v[q] = p[st * q];
     mag = max(mag, fx_mag(v[q]));
   }
-  const int E = fx_exponent(mag);
+  E = fx_exponent(mag);
 #pragma unroll
   for (int q = 0; q < N; ++q) fx_split(v[q], E, h[q], l[q]);
-  f(E);
-  return fx_bad(mag);
+  if (mag == 0u) {  // zeros, or values so small that their high words are
+    unsigned low = 0u;
+#pragma unroll 1
+    for (int q = 0; q < N; ++q) low |= (unsigned)__double2loint(p[st * q]);
+    return low == 0u;
+  }
+  return !fx_bad(mag);
+}
+
+// out = M in along a line without a scale, in FP64: M = D, or D^T.  in and out may be the same line.
+template <int N>
+__device__ __noinline__ void ax_slow_line(const double* D, bool transposed, const double* in, double* out, int st) {
+  double v[N];
+#pragma unroll
+  for (int q = 0; q < N; ++q) v[q] = in[st * q];
+#pragma unroll 1
+  for (int k = 0; k < N; ++k) {
+    double acc = 0.0;
+#pragma unroll
+    for (int q = 0; q < N; ++q) acc = fma(D[transposed ? q * N + k : k * N + q], v[q], acc);
+    out[st * k] = acc;
+  }
 }
 
 template <int N>
 struct AxFxDims {
   static constexpr int NP = N % 2 ? N : N + 1;     // padded row: odd, so 8-byte lines do not conflict
   static constexpr int PLANE = NP * N, VOL = NP * N * N;
+  // scales of the r- and s-lines of w: even N in the padding of R's and S's rows, odd N behind the arrays
+  static constexpr int SIZE = 3 * VOL + (N % 2 ? (2 * N * N + 1) / 2 : 0);  // doubles per element
 };
+
+constexpr int FX_NO_SCALE = INT_MAX;  // of a line whose results are doubles
+
+// Scale of line (c, k) of an array's N^2 lines, c the coordinate across and k = 0 .. N - 1 the plane.
+template <int N>
+__device__ __forceinline__ int* ax_line_scale(double* U, int array, int c, int k) {
+  using Dm = AxFxDims<N>;
+  if constexpr (N % 2) return reinterpret_cast<int*>(U + 3 * Dm::VOL) + (array - 1) * N * N + c + N * k;
+  else return reinterpret_cast<int*>(U + array * Dm::VOL + Dm::NP * c + Dm::PLANE * k + N);
+}
 
 // A column's place in the lattice (FOLD): its element and its Dirichlet points (bit k).
 struct AxLattice {
@@ -102,57 +138,6 @@ __device__ __forceinline__ double ax_fx_input(const AxFxArgs& a, int64_t gi, boo
   return zero ? 0.0 : v;
 }
 
-// A_L u of the block's elements in FP64, columns of results to U (the caller's column of each
-// thread).  Every thread of the block calls it.
-template <int N>
-__device__ __noinline__ void ax_slow_block(const AxFxArgs& a, int64_t e, bool valid, int i, int j, unsigned zmask,
-                                           double* U, double* R, double* S) {
-  constexpr int N2 = N * N, NP = AxFxDims<N>::NP, PL = AxFxDims<N>::PLANE;
-  const int64_t eb = e * (N2 * N) + i + N * j;
-  double* Uc = U + i + NP * j;
-  __syncthreads();
-  if (valid) {
-#pragma unroll 1
-    for (int k = 0; k < N; ++k) Uc[PL * k] = ax_fx_input(a, eb + N2 * k, (zmask >> k) & 1u);
-  }
-  __syncthreads();
-  double ry[N];
-#pragma unroll
-  for (int l = 0; l < N; ++l) ry[l] = 0.0;
-  if (valid) {
-#pragma unroll 1
-    for (int k = 0; k < N; ++k) {
-      double ur = 0.0, us = 0.0, ut = 0.0;
-#pragma unroll 1
-      for (int l = 0; l < N; ++l) {
-        ur = fma(a.D[i * N + l], U[l + NP * j + PL * k], ur);
-        us = fma(a.D[j * N + l], U[i + NP * l + PL * k], us);
-        ut = fma(a.D[k * N + l], Uc[PL * l], ut);
-      }
-      const double* g = a.G + eb + N2 * k;
-      const double grr = g[0], grs = g[a.L], grt = g[2 * a.L], gss = g[3 * a.L], gst = g[4 * a.L], gtt = g[5 * a.L];
-      R[i + NP * j + PL * k] = fma(grt, ut, fma(grs, us, grr * ur));
-      S[i + NP * j + PL * k] = fma(gst, ut, fma(gss, us, grs * ur));
-      const double wt = fma(gtt, ut, fma(gst, us, grt * ur));
-#pragma unroll
-      for (int l = 0; l < N; ++l) ry[l] = fma(a.D[k * N + l], wt, ry[l]);
-    }
-  }
-  __syncthreads();
-  if (valid) {
-#pragma unroll
-    for (int k = 0; k < N; ++k) {
-      double acc = ry[k];
-#pragma unroll 1
-      for (int l = 0; l < N; ++l) {
-        acc = fma(a.D[l * N + i], R[l + NP * j + PL * k], acc);
-        acc = fma(a.D[l * N + j], S[i + NP * l + PL * k], acc);
-      }
-      Uc[PL * k] = acc;
-    }
-  }
-}
-
 // Registers: the kernel waits on memory, shared memory and dependent integer operations in turn, so
 // resident warps are worth more than registers up to the point where lines spill.
 template <int N>
@@ -160,22 +145,20 @@ constexpr int ax_fx_regs() { return N <= 9 ? 64 : (N == 10 ? 72 : 96); }
 
 template <int N, bool FOLD>
 __global__ void __maxnreg__(ax_fx_regs<N>())
-    ax_fx_kernel(const __grid_constant__ AxFxArgs a, const __grid_constant__ FxFold<N, N> tD,
+    ax_fx_kernel(const __grid_constant__ AxFxArgs a, const __grid_constant__ FxFoldRows<N, N> tD,
                  const __grid_constant__ FxFold<N, N> tT) {
   constexpr int N2 = N * N, N3 = N2 * N, NP = AxFxDims<N>::NP, PL = AxFxDims<N>::PLANE, VOL = AxFxDims<N>::VOL;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int le = threadIdx.x / N2;
   const int t = threadIdx.x - le * N2;
   const int i = t % N, j = t / N;  // the thread's column; also (j, k) of its r-line, (i, k) of its s-line
-  double* U = reinterpret_cast<double*>(smem_raw) + (size_t)le * 3 * VOL;
+  double* U = reinterpret_cast<double*>(smem_raw) + (size_t)le * AxFxDims<N>::SIZE;
   double* R = U + VOL;
   double* S = R + VOL;
-  unsigned* mags = reinterpret_cast<unsigned*>(reinterpret_cast<double*>(smem_raw) + (size_t)a.NE * 3 * VOL);
   const int64_t e = (int64_t)blockIdx.x * a.NE + le;
   const bool valid = e < a.E;
   const int64_t eb = e * N3 + t;
   const int col = i + NP * j, rl = NP * i + PL * j, sl = i + PL * j;  // lines: column, (j=i,k=j), (i,k=j)
-  if (t == 0) mags[le] = 0u;
   // the column's place in the lattice (E < 2^31): needed last, worth registers until then for small N
   constexpr bool EARLY = FOLD && N < 8;
   AxLattice at{};
@@ -191,93 +174,99 @@ __global__ void __maxnreg__(ax_fx_regs<N>())
         if (!(a.pflag[eb + N2 * k] & PF_FREE)) zin |= 1u << k;
     }
   }
-  bool bad = false;
-  int Et;  // scale of the thread's column
-  {
-    unsigned mag = 0u;
 #pragma unroll
-    for (int k = 0; k < N; ++k) {
-      const double v = valid ? ax_fx_input(a, eb + N2 * k, (zin >> k) & 1u) : 0.0;
-      U[col + PL * k] = v;
-      mag = max(mag, fx_mag(v));
-    }
-    bad = fx_bad(mag);
-    Et = fx_exponent(mag);
-  }
+  for (int k = 0; k < N; ++k) U[col + PL * k] = valid ? ax_fx_input(a, eb + N2 * k, (zin >> k) & 1u) : 0.0;
   __syncthreads();
+  // a line of doubles contracted on its own scale, st apart: in and out may be the same line
+  auto contract = [&](const FxFoldRows<N, N>& m, bool transposed, const double* in, double* out, int st) {
+    int h[N], l[N], E;
+    if (fx_split_line<N>(in, st, h, l, E))
+      fx_contract<N, N, -1>(m, h, l, [&](int q, long long r) { out[st * q] = fx_double(r, E - m.row_k(q)); });
+    else
+      ax_slow_line<N>(a.D, transposed, in, out, st);
+  };
   // r-lines and s-lines
-  {
-    int h[N], l[N];
-    bad |= fx_split_line<N>(U + rl, 1, h, l, [&](int E) {
-      fx_contract<N, N, -1>(tD, h, l, [&](int q, long long r) { R[rl + q] = fx_double(r, E - tD.k); });
-    });
-    bad |= fx_split_line<N>(U + sl, NP, h, l, [&](int E) {
-      fx_contract<N, N, -1>(tD, h, l, [&](int q, long long r) { S[sl + NP * q] = fx_double(r, E - tD.k); });
-    });
-  }
-  bad = __syncthreads_or(bad);
-  if (!bad) {
-    // t-lines and the pointwise factors: the thread's column.  From N = 8 the factors have a loop of
-    // their own, two points at a time behind a barrier (which the compiler does not move loads across),
-    // so that the contraction and the loads in flight do not compete for registers: p = 7 429 -> 406 us,
-    // p = 8 192 -> 182, p = 9 283 -> 271; p = 5 and 6 are 8% faster fused (198, 138)
-    constexpr bool SPLIT = N >= 8;
-    unsigned mag = 0u;
-    const double* g = a.G + (valid ? eb : (int64_t)t);
-    auto pointwise = [&](int q, double ut) {
-      const double* gq = g + N2 * q;
-      const double grr = gq[0], grs = gq[a.L], grt = gq[2 * a.L], gss = gq[3 * a.L], gst = gq[4 * a.L], gtt = gq[5 * a.L];
-      const double ur = R[col + PL * q], us = S[col + PL * q];
-      const double wr = fma(grt, ut, fma(grs, us, grr * ur));
-      const double ws = fma(gst, ut, fma(gss, us, grs * ur));
-      const double wt = fma(gtt, ut, fma(gst, us, grt * ur));
-      R[col + PL * q] = wr;
-      S[col + PL * q] = ws;
-      U[col + PL * q] = wt;
-      mag = max(max(mag, fx_mag(wr)), max(fx_mag(ws), fx_mag(wt)));
-    };
-    {
-      const int eb1 = Et - tD.k;
-      int h[N], l[N];
-#pragma unroll
-      for (int q = 0; q < N; ++q) fx_split(U[col + PL * q], Et, h[q], l[q]);
-      fx_contract<N, N, -1>(tD, h, l, [&](int q, long long r) {
-        const double ut = fx_double(r, eb1);
-        if constexpr (SPLIT) U[col + PL * q] = ut;
-        else pointwise(q, ut);
-      });
-    }
-    if constexpr (SPLIT) {
-      __syncthreads();
+  contract(tD, false, U + rl, R + rl, 1);
+  contract(tD, false, U + sl, S + sl, NP);
+  __syncthreads();
+  // t-lines and the pointwise factors: the thread's column.  From N = 8 the factors have a loop of
+  // their own, two points at a time behind a barrier (which the compiler does not move loads across),
+  // so that the contraction and the loads in flight do not compete for registers: p = 7 429 -> 406 us,
+  // p = 8 192 -> 182, p = 9 283 -> 271; p = 5 and 6 are 8% faster fused (198, 138)
+  constexpr bool SPLIT = N >= 8;
+  const double* g = a.G + (valid ? eb : (int64_t)t);
+  auto pointwise = [&](int q, double ut) {
+    const double* gq = g + N2 * q;
+    const double grr = gq[0], grs = gq[a.L], grt = gq[2 * a.L], gss = gq[3 * a.L], gst = gq[4 * a.L], gtt = gq[5 * a.L];
+    const double ur = R[col + PL * q], us = S[col + PL * q];
+    R[col + PL * q] = fma(grt, ut, fma(grs, us, grr * ur));
+    S[col + PL * q] = fma(gst, ut, fma(gss, us, grs * ur));
+    U[col + PL * q] = fma(gtt, ut, fma(gst, us, grt * ur));
+  };
+  if constexpr (SPLIT) {
+    contract(tD, false, U + col, U + col, PL);
+    __syncthreads();
 #pragma unroll 2
+    for (int q = 0; q < N; ++q) pointwise(q, U[col + PL * q]);
+  } else {
+    int h[N], l[N], E;
+    if (fx_split_line<N>(U + col, PL, h, l, E)) {
+      fx_contract<N, N, -1>(tD, h, l, [&](int q, long long r) { pointwise(q, fx_double(r, E - tD.row_k(q))); });
+    } else {
+      ax_slow_line<N>(a.D, false, U + col, U + col, PL);
+#pragma unroll 1
       for (int q = 0; q < N; ++q) pointwise(q, U[col + PL * q]);
     }
-    if (mag) atomicMax(&mags[le], mag);
-    __syncthreads();
-    const unsigned mag2 = mags[le];
-    const int E2 = fx_exponent(mag2);
-    {
-      int h[N], l[N];
-#pragma unroll
-      for (int q = 0; q < N; ++q) fx_split(R[rl + q], E2, h[q], l[q]);
-      fx_contract<N, N, -1>(tT, h, l, [&](int q, long long r) { reinterpret_cast<long long*>(R)[rl + q] = r; });
-#pragma unroll
-      for (int q = 0; q < N; ++q) fx_split(S[sl + NP * q], E2, h[q], l[q]);
-      fx_contract<N, N, -1>(tT, h, l, [&](int q, long long r) { reinterpret_cast<long long*>(S)[sl + NP * q] = r; });
+  }
+  __syncthreads();
+  // r-lines and s-lines of w, in place: 64-bit integers on the line's own scale, or the doubles of a line
+  // without one
+  auto transposed = [&](double* w, int st) {
+    int h[N], l[N], E;
+    if (fx_split_line<N>(w, st, h, l, E)) {
+      fx_contract<N, N, -1>(tT, h, l, [&](int q, long long r) { reinterpret_cast<long long*>(w)[st * q] = r; });
+    } else {
+      ax_slow_line<N>(a.D, true, w, w, st);
+      E = FX_NO_SCALE;
     }
-    bad = __syncthreads_or(fx_bad(mag2));
-    if (!bad) {
-      const int eb2 = E2 - tT.k;
-      int h[N], l[N];
-#pragma unroll
-      for (int q = 0; q < N; ++q) fx_split(U[col + PL * q], E2, h[q], l[q]);
+    return E;
+  };
+  const int Er = transposed(R + rl, 1), Es = transposed(S + sl, NP);
+  *ax_line_scale<N>(U, 1, i, j) = Er;
+  *ax_line_scale<N>(U, 2, i, j) = Es;
+  const bool slow = __syncthreads_or(max(Er, Es) == FX_NO_SCALE);
+  // t-lines; the three parts are added on the largest of their scales (what a smaller one loses there is
+  // below 2^-60 of the sum's largest part) and rounded to double once
+  {
+    int h[N], l[N], E;
+    const bool scaled = fx_split_line<N>(U + col, PL, h, l, E);
+    auto sum = [&](int q, long long r, int er, int es) {
+      const int m = max(E, max(er, es));
+      r = fx_shr(r, m - E) + fx_shr(reinterpret_cast<const long long*>(R)[col + PL * q], m - er) +
+          fx_shr(reinterpret_cast<const long long*>(S)[col + PL * q], m - es);
+      return fx_double(r, m - tT.k);
+    };
+    if (scaled && !slow) {
       fx_contract<N, N, -1>(tT, h, l, [&](int q, long long r) {
-        r += reinterpret_cast<const long long*>(R)[col + PL * q] + reinterpret_cast<const long long*>(S)[col + PL * q];
-        U[col + PL * q] = fx_double(r, eb2);
+        U[col + PL * q] = sum(q, r, *ax_line_scale<N>(U, 1, j, q), *ax_line_scale<N>(U, 2, i, q));
       });
+    } else {
+      if (scaled)
+        fx_contract<N, N, -1>(tT, h, l, [&](int q, long long r) { reinterpret_cast<long long*>(U)[col + PL * q] = r; });
+      else
+        ax_slow_line<N>(a.D, true, U + col, U + col, PL);
+      auto value = [&](const double* p, int e) {
+        return e == FX_NO_SCALE ? *p : fx_double(*reinterpret_cast<const long long*>(p), e - tT.k);
+      };
+#pragma unroll 1
+      for (int q = 0; q < N; ++q) {
+        const int er = *ax_line_scale<N>(U, 1, j, q), es = *ax_line_scale<N>(U, 2, i, q);
+        double* u = U + col + PL * q;
+        if (scaled && max(er, es) != FX_NO_SCALE) *u = sum(q, *reinterpret_cast<const long long*>(u), er, es);
+        else *u = value(u, scaled ? E : FX_NO_SCALE) + (value(R + col + PL * q, er) + value(S + col + PL * q, es));
+      }
     }
   }
-  if (bad) ax_slow_block<N>(a, e, valid, i, j, zin, U, R, S);
   // U: A_L u, each thread's own column
   if constexpr (FOLD) {
     // residual form: each copy's b / multiplicity - (A_L u); a copy on an interior interface
@@ -312,8 +301,8 @@ __global__ void __maxnreg__(ax_fx_regs<N>())
       const int lp = idx / N2, jk = idx - lp * N2;
       const int el = (int)(e0 + lp);
       if (el + 1 < a.E && el % a.nx < a.nx - 1) {
-        double* p = reinterpret_cast<double*>(smem_raw) + (size_t)lp * 3 * VOL + NP * jk + N - 1;
-        double* q = p + 3 * VOL - (N - 1);
+        double* p = reinterpret_cast<double*>(smem_raw) + (size_t)lp * AxFxDims<N>::SIZE + NP * jk + N - 1;
+        double* q = p + AxFxDims<N>::SIZE - (N - 1);
         const double v = *p + *q;
         *p = v;
         *q = v;
@@ -358,8 +347,9 @@ __global__ void gs_fold_fixup_x(int64_t E, int NE, int nx, double* __restrict__ 
 
 template <int N>
 struct AxFxTables {
-  FxFold<N, N> D, T;  // three results of T = D^T are added in 64 bits
-  explicit AxFxTables(const double* d) : D(fx_fold_tables<N, N>(d, -1, 60)) {
+  FxFoldRows<N, N> D;
+  FxFold<N, N> T;  // D^T: three results are added in 64 bits
+  explicit AxFxTables(const double* d) : D(fx_fold_rows<N, N>(d, -1)) {
     double t[N * N];
     for (int r = 0; r < N; ++r)
       for (int c = 0; c < N; ++c) t[r * N + c] = d[c * N + r];
@@ -370,7 +360,7 @@ struct AxFxTables {
 template <int N>
 static int launch_ax_fx(const Level& lv, const double* u, double* y, bool mask_in, const double* sub,
                         const double* dinv, int NE, bool fold, cudaStream_t s) {
-  static_assert(sizeof(FxFold<N, N>) <= 1536, "two folded tables and the arguments fit the 4 KB of parameters");
+  static_assert(sizeof(FxFoldRows<N, N>) <= 1536, "two folded tables and the arguments fit the 4 KB of parameters");
   // the tables depend on the order only: formed once per process
   static const AxFxTables<N> tab(lv.basis.D);
   AxFxArgs a{};
@@ -386,7 +376,7 @@ static int launch_ax_fx(const Level& lv, const double* u, double* y, bool mask_i
   a.y = y;
   a.mask_in = mask_in;
   const int threads = NE * N * N;
-  const size_t smem = (size_t)NE * (3 * AxFxDims<N>::VOL * sizeof(double) + sizeof(unsigned));
+  const size_t smem = (size_t)NE * AxFxDims<N>::SIZE * sizeof(double);
   const unsigned blocks = (unsigned)((lv.E + NE - 1) / NE);
   if (fold) {
     a.nx = lv.nel[0];
