@@ -3,26 +3,32 @@
 // element by element (transfer.cu adds QQ^T on the coarse level).  Both GLL point sets are symmetric
 // about 0, so J is centro-symmetric and its lines fold.
 //
-// Each thread takes one line per direction and contracts it on the line's own scale.  The first
-// direction's line is read straight from memory (NI consecutive values); its results, and the second
-// direction's, are kept in shared memory as 64-bit integers on a scale common to the element, which
-// starts from the element's largest value and then only takes the fixed bound of a contraction
-// (|R| < 2^62): interpolation hardly changes magnitudes, so no renormalisation by value is needed.
-// The last direction leaves as doubles, stored from its lines (a warp's lanes hold consecutive
-// (a, b): each plane of an element is a contiguous store).
+// Each thread takes one line per direction and contracts it on the line's own scale; between the
+// directions the values are doubles in shared memory.  The first direction's line is read straight
+// from memory (NI consecutive values), the last direction's results are stored from its lines (a
+// warp's lanes hold consecutive (a, b): each plane of an element is a contiguous store).
+//
+// The two point sets share their end points (and for two odd counts the middle one), where J's rows are
+// unit vectors: prolongation copies those values and contracts the others; restriction adds them to
+// their one result and contracts the inner points only.  So a value is never cut on the scale of values
+// that do not enter its result, and a face of the prolonged vector depends on the face's values
+// alone: both copies of an interface point get the same bits.
 //
 // Measured on GB300 (us per launch, restriction / prolongation; in brackets the FP64 kernels this one
-// replaced, bound by the FP64 pipe): 32^3 elements p = 7 -> 5 96 / 86 [346 / 383], 5 -> 3 40 / 35
-// [117 / 127], 3 -> 1 13 / 12 [23 / 25]; 20^3 9 -> 5 48 / 42 [135 / 140]; even orders (not folded
-// before) 20^3 8 -> 4 34 / 29.  Memory needs 33 us of the 96; the rest is integer issue.
+// replaced, bound by the FP64 pipe): 32^3 elements p = 7 -> 5 99 / 88 [346 / 383], 5 -> 3 41 / 34
+// [117 / 127], 3 -> 1 13 / 11 [23 / 25]; 20^3 9 -> 5 50 / 43 [135 / 140]; even orders (not folded
+// before) 20^3 8 -> 4 33 / 27.  Memory needs 33 us of the 99; the rest is integer issue.  64-bit
+// integers on the element's scale between the directions were 0 to 6% faster (96 / 86, 40 / 35), but
+// cut every value on its element's largest one, and left the copies of an interface point
+// unequal.
 //
-// Error against extended precision (2-norm) over the FP64 contraction's: 0.35 to 0.75 for random and
-// smooth values, 0.7 to 2.7 for values that decay by eight decades across the element.  One scale per
-// element for all three directions needed 40% fewer integer operations, but was 1.4 to 2.6 times less
-// exact than FP64 in the restriction.
+// Error against extended precision (2-norm, host emulation), over the FP64 contraction's: 0.43 to 0.89
+// for random values, 0.40 to 1.0 for smooth ones, 0.33 to 0.78 for values that decay by eight decades
+// across the element, 0.28 to 1.01 around one value 10^8 times the others (2 -> 1, whose rows have two
+// entries of 1/2: 1.0 to 1.19, the conversion rounds ties upwards).
 //
-// Elements without a common scale (infinities, NaN, magnitudes at the ends of the range) send their
-// block to transfer_slow_block, the same contraction in FP64.
+// A line without a scale (infinities, NaN, magnitudes at the ends of the range) is contracted in FP64 by
+// itself.
 #include "fxp.h"
 #include "reduce.h"
 #include "se_internal.h"
@@ -46,21 +52,25 @@ struct TransferFxDims {
   static constexpr int THREADS = (NE * MOST + 31) / 32 * 32;
   static constexpr int RB = NO % 2 ? NO : NO + 1;   // row stride of the first result
   static constexpr int B = RB * NI * NI, A = NO * NO * NI;
-  static constexpr size_t SMEM = (size_t)NE * ((A + B) * 8 + 8);
+  static constexpr size_t SMEM = (size_t)NE * (A + B) * 8;
+  // what is contracted: prolongation all inputs to the inner outputs, restriction the inner inputs
+  static constexpr int I0 = RESTRICT ? 1 : 0, O0 = RESTRICT ? 0 : 1, NL = NI - 2 * I0, NR = NO - 2 * O0;
+  static constexpr bool MID = NI % 2 == 1 && NO % 2 == 1;  // a middle point in common
 };
 
-// The line operator: J, or J^T for the restriction (host).
+// The line operator without its unit rows: rows of J, or columns of J^T for the restriction (host).
 template <int NF, int NC, bool RESTRICT>
-using TransferFxTable = FxFold<TransferFxDims<NF, NC, RESTRICT>::NO, TransferFxDims<NF, NC, RESTRICT>::NI>;
+using TransferFxTable = FxFold<TransferFxDims<NF, NC, RESTRICT>::NR, TransferFxDims<NF, NC, RESTRICT>::NL>;
 
 template <int NF, int NC, bool RESTRICT>
 static TransferFxTable<NF, NC, RESTRICT> transfer_fx_table() {
   using D = TransferFxDims<NF, NC, RESTRICT>;
-  double J[NF * NC], M[NF * NC];
+  double J[NF * NC], M[D::NR * D::NL];
   interp_matrix(NF - 1, NC - 1, J);
-  for (int o = 0; o < D::NO; ++o)
-    for (int i = 0; i < D::NI; ++i) M[o * D::NI + i] = RESTRICT ? J[i * NC + o] : J[o * NC + i];
-  return fx_fold_tables<D::NO, D::NI>(M, 1, 60);
+  for (int o = 0; o < D::NR; ++o)
+    for (int i = 0; i < D::NL; ++i)
+      M[o * D::NL + i] = RESTRICT ? J[(i + D::I0) * NC + o] : J[(o + D::O0) * NC + i];
+  return fx_fold_tables<D::NR, D::NL>(M, 1, 60);
 }
 
 __device__ __forceinline__ double transfer_fx_input(const TransferFxArgs& a, int64_t gi, bool weighted) {
@@ -69,40 +79,48 @@ __device__ __forceinline__ double transfer_fx_input(const TransferFxArgs& a, int
   return v;
 }
 
-template <int NF, int NC, bool RESTRICT>
-__device__ __noinline__ void transfer_slow_block(const TransferFxArgs& a, int64_t e0, int ne, double* bufA, double* bufB) {
+// out(o, value) of the line v, on its own scale; false where it has none.
+template <int NF, int NC, bool RESTRICT, class Out>
+__device__ __forceinline__ bool transfer_fx_line(const TransferFxTable<NF, NC, RESTRICT>& m,
+                                                 const double (&v)[TransferFxDims<NF, NC, RESTRICT>::NI], Out&& out) {
   using D = TransferFxDims<NF, NC, RESTRICT>;
-  constexpr int NI = D::NI, NO = D::NO;
-  auto m = [&](int o, int i) { return RESTRICT ? a.J[i * NC + o] : a.J[o * NC + i]; };
-  __syncthreads();
-#pragma unroll 1
-  for (int q = threadIdx.x; q < ne * NO * D::L1; q += blockDim.x) {
-    const int le = q / (NO * D::L1), r = q - le * NO * D::L1, o = r % NO, jk = r / NO;
-    double acc = 0.0;
-#pragma unroll 1
-    for (int i = 0; i < NI; ++i)
-      acc = fma(m(o, i), transfer_fx_input(a, (e0 + le) * (NI * NI * NI) + i + NI * jk, RESTRICT), acc);
-    bufB[le * D::B + o + D::RB * jk] = acc;
+  constexpr int NI = D::NI, NO = D::NO, NL = D::NL;
+  // the value that only adds to its own result
+  auto apart = [](int i) { return RESTRICT && D::MID && i == NI / 2; };
+  unsigned mag = 0u, rest = 0u;
+#pragma unroll
+  for (int i = 0; i < NI; ++i) {
+    const bool in = i >= D::I0 && i < NI - D::I0 && !apart(i);
+    (in ? mag : rest) = max(in ? mag : rest, fx_mag(v[i]));
   }
-  __syncthreads();
-#pragma unroll 1
-  for (int q = threadIdx.x; q < ne * NO * D::L2; q += blockDim.x) {
-    const int le = q / (NO * D::L2), r = q - le * NO * D::L2, x = r % NO, b = (r / NO) % NO, k = r / (NO * NO);
-    double acc = 0.0;
-#pragma unroll 1
-    for (int j = 0; j < NI; ++j) acc = fma(m(b, j), bufB[le * D::B + x + D::RB * (j + NI * k)], acc);
-    bufA[le * D::A + x + NO * (b + NO * k)] = acc;
+  if (fx_bad(mag) || fx_bad(max(mag, rest))) return false;
+  if (mag == 0u) {  // zeros, or values so small that their high words are
+    unsigned low = 0u;
+#pragma unroll
+    for (int i = D::I0; i < NI - D::I0; ++i) low |= (unsigned)__double2loint(v[i]);
+    if (low != 0u) return false;
   }
-  __syncthreads();
-#pragma unroll 1
-  for (int q = threadIdx.x; q < ne * NO * D::L3; q += blockDim.x) {
-    const int le = q / (NO * D::L3), r = q - le * NO * D::L3, ab = r % D::L3, c = r / D::L3;
-    double acc = 0.0;
-#pragma unroll 1
-    for (int k = 0; k < NI; ++k) acc = fma(m(c, k), bufA[le * D::A + ab + D::L3 * k], acc);
-    double* out = a.out + (e0 + le) * (NO * NO * NO) + r;
-    *out = a.accumulate ? *out + acc : acc;
+  const int E = fx_exponent(mag);
+  int h[NL], l[NL];
+#pragma unroll
+  for (int i = 0; i < NL; ++i) {
+    fx_split(v[i + D::I0], E, h[i], l[i]);
+    if (apart(i + D::I0)) h[i] = l[i] = 0;
   }
+  if constexpr (!RESTRICT) {
+    out(0, v[0]);
+    out(NO - 1, v[NI - 1]);
+    if constexpr (D::MID) out(NO / 2, v[NI / 2]);
+  }
+  fx_contract<D::NR, NL, 1>(m, h, l, [&](int q, long long r) {
+    const int o = q + D::O0;
+    const double w = fx_double(r, E - m.k);
+    if (RESTRICT && o == 0) out(o, w + v[0]);
+    else if (RESTRICT && o == NO - 1) out(o, w + v[NI - 1]);
+    else if (RESTRICT && D::MID && o == NO / 2) out(o, w + v[NI / 2]);
+    else if (!(!RESTRICT && D::MID && o == NO / 2)) out(o, w);
+  });
+  return true;
 }
 
 template <int NF, int NC, bool RESTRICT>
@@ -112,68 +130,43 @@ __global__ void __launch_bounds__(TransferFxDims<NF, NC, RESTRICT>::THREADS)
   using D = TransferFxDims<NF, NC, RESTRICT>;
   constexpr int NI = D::NI, NO = D::NO, NE = D::NE;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  long long* bufB = reinterpret_cast<long long*>(smem_raw);  // first direction's results
-  long long* bufA = bufB + NE * D::B;                         // second direction's
-  unsigned* mags = reinterpret_cast<unsigned*>(bufA + NE * D::A);
+  double* bufB = reinterpret_cast<double*>(smem_raw);  // first direction's results
+  double* bufA = bufB + NE * D::B;                     // second direction's
   const int tid = threadIdx.x;
   const int64_t e0 = (int64_t)blockIdx.x * NE;
   const int ne = (int)(a.E - e0 < NE ? a.E - e0 : NE);
-  if (tid < NE) mags[tid] = 0u;
-  __syncthreads();
-  int h[NI], l[NI];
+  // a line: in(i) read once, results to out(o, value)
+  auto line = [&](auto&& in, auto&& out) {
+    double v[NI];
+#pragma unroll
+    for (int i = 0; i < NI; ++i) v[i] = in(i);
+    if (!transfer_fx_line<NF, NC, RESTRICT>(m, v, out)) {
+#pragma unroll 1
+      for (int o = 0; o < NO; ++o) {
+        double acc = 0.0;
+#pragma unroll
+        for (int i = 0; i < NI; ++i) acc = fma(RESTRICT ? a.J[i * NC + o] : a.J[o * NC + i], v[i], acc);
+        out(o, acc);
+      }
+    }
+  };
   // ---- direction r: lines (j, k)
-  bool bad = false;
   {
     const int le = tid / D::L1, jk = tid - le * D::L1;
-    const bool on = le < ne;
-    int E = FX_EMIN;
-    if (on) {
-      double v[NI];
-      unsigned mag = 0u;
-#pragma unroll
-      for (int i = 0; i < NI; ++i) {
-        v[i] = transfer_fx_input(a, (e0 + le) * (NI * NI * NI) + i + NI * jk, RESTRICT);
-        mag = max(mag, fx_mag(v[i]));
-      }
-      if (mag) atomicMax(mags + le, mag);
-      bad = fx_bad(mag);
-      E = fx_exponent(mag);
-#pragma unroll
-      for (int i = 0; i < NI; ++i) fx_split(v[i], E, h[i], l[i]);
-    }
-    __syncthreads();
-    if (on) {
-      const int back = fx_exponent(mags[le]) - E;
-      long long* B = bufB + le * D::B + D::RB * jk;
-      fx_contract<NO, NI, 1>(m, h, l, [&](int o, long long r) { B[o] = fx_shr(r, back); });
+    if (le < ne) {
+      double* B = bufB + le * D::B + D::RB * jk;
+      line([&](int i) { return transfer_fx_input(a, (e0 + le) * (NI * NI * NI) + i + NI * jk, RESTRICT); },
+           [&](int o, double w) { B[o] = w; });
     }
   }
-  bad = __syncthreads_or(bad);
-  if (bad) {
-    transfer_slow_block<NF, NC, RESTRICT>(a, e0, ne, reinterpret_cast<double*>(bufA), reinterpret_cast<double*>(bufB));
-    return;
-  }
-  // a line of results on its own scale: R 2^n / 2^6
-  auto line = [&](const long long* p, int st) {
-    unsigned high = 0u;
-    long long r[NI];
-#pragma unroll
-    for (int i = 0; i < NI; ++i) {
-      r[i] = p[st * i];
-      high = max(high, fx_high(r[i]));
-    }
-    const int n = fx_norm(high);
-#pragma unroll
-    for (int i = 0; i < NI; ++i) fx_renorm(r[i], n, h[i], l[i]);
-    return n;
-  };
-  // ---- direction s: lines (a, k); |R| < 2^62 needs n >= 1, the common scale is that of n = 1
+  __syncthreads();
+  // ---- direction s: lines (a, k)
   {
     const int le = tid / D::L2, r2 = tid - le * D::L2, k = r2 / NO, x = r2 - k * NO;
     if (le < ne) {
-      const int back = line(bufB + le * D::B + x + D::RB * NI * k, D::RB) - 1;
-      long long* A = bufA + le * D::A + x + D::L3 * k;
-      fx_contract<NO, NI, 1>(m, h, l, [&](int o, long long r) { A[NO * o] = fx_shr(r, back); });
+      const double* B = bufB + le * D::B + x + D::RB * NI * k;
+      double* A = bufA + le * D::A + x + D::L3 * k;
+      line([&](int i) { return B[D::RB * i]; }, [&](int o, double w) { A[NO * o] = w; });
     }
   }
   __syncthreads();
@@ -181,14 +174,10 @@ __global__ void __launch_bounds__(TransferFxDims<NF, NC, RESTRICT>::THREADS)
   {
     const int le = tid / D::L3, ab = tid - le * D::L3;
     if (le < ne) {
-      const int n = line(bufA + le * D::A + ab, D::L3);
-      // x in units 2^(E - 1079) gives R in units 2^(E - 1023 - k); R 2^n / 2^6 has E + 62 - n - k
-      const int eb = fx_exponent(mags[le]) - m.k + 61 - m.k + 62 - n - m.k;
+      const double* A = bufA + le * D::A + ab;
       double* out = a.out + (e0 + le) * (NO * NO * NO) + ab;
-      fx_contract<NO, NI, 1>(m, h, l, [&](int o, long long r) {
-        const double v = fx_double(r, eb);
-        out[D::L3 * o] = a.accumulate ? out[D::L3 * o] + v : v;
-      });
+      line([&](int i) { return A[D::L3 * i]; },
+           [&](int o, double w) { out[D::L3 * o] = a.accumulate ? out[D::L3 * o] + w : w; });
     }
   }
 }

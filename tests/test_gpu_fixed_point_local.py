@@ -66,3 +66,120 @@ def test_operator_elements_do_not_share_a_fallback(p, value):
     finally:
         se.se_tune_set(p, se.SE_FP64, 0, 0)
         c.close()
+
+
+def _transfer(c, pf, pc):
+    se = c.se
+    P = se.se_pmg_setup(c.m, se.pmg_desc((pf, pc, 1) if pc > 1 else (pf, 1), se.SE_SMOOTH_JACOBI, 1))
+    return P, o.make_level(c.V, c.nel, pc, c.lv.bc, c.amp)
+
+
+PAIRS = [(2, 1), (3, 1), (3, 2), (4, 2), (5, 3), (6, 4), (7, 5), (8, 4), (9, 5), (10, 4), (10, 9), (10, 1)]
+
+
+@pytest.mark.parametrize("pf,pc", PAIRS)
+def test_prolongation_is_continuous_to_the_last_bit(pf, pc):
+    """Every copy of an interface point depends on the interface's values alone, by the same operations."""
+    c = Case((4, 3, 3), pf, seed=23, bc=("D", "N", "N", "D", "N", "N"))
+    try:
+        P, lc = _transfer(c, pf, pc)
+        ef = c.empty()
+        c.se.se_pmg_prolong(P, 0, c.to_gpu(c.random_continuous(8, lv=lc) * np.exp(3.0)), ef)
+        got = c.to_np(ef)
+        one = np.zeros(c.lv.n_global)
+        one[c.lv.gid] = got
+        assert np.array_equal(one[c.lv.gid].view(np.int64), got.view(np.int64))
+        c.se.se_pmg_destroy(P)
+    finally:
+        c.close()
+
+
+@pytest.mark.parametrize("pf,pc", PAIRS)
+@pytest.mark.parametrize("spike", [1e4, 1e12])
+def test_transfers_away_from_a_large_value(pf, pc, spike):
+    """A large value at an element's corner: J's unit rows keep it from the faces opposite to it in the
+    prolongation, and from everything but its own node in the restriction; likewise a large value in
+    the element's middle where both orders have that point."""
+    c = Case((3, 2, 2), pf, seed=24, bc=("N",) * 6)
+    try:
+        P, lc = _transfer(c, pf, pc)
+        rng = np.random.default_rng(pf)
+        ec = rng.uniform(-1, 1, lc.gid.shape)
+        ec[4, 0, 0, 0] = 0.0
+        ref = o.prolong(c.lv, lc, ec)[4]
+        ec[4, 0, 0, 0] = spike
+        ef, rc = c.empty(), c.empty(lc.gid.size)
+        c.se.se_pmg_prolong(P, 0, c.to_gpu(ec), ef)
+        got = c.to_np(ef)[4]
+        far = np.zeros(got.shape, bool)
+        far[-1], far[:, -1], far[:, :, -1] = True, True, True
+        assert np.max(np.abs(got - ref)[far]) <= 1e-13 * np.max(np.abs(ref[far]))
+        places = [(0, 0, 0)] + ([(pf // 2,) * 3] if pf % 2 == 0 and pc % 2 == 0 else [])
+        for at in places:
+            rf = rng.uniform(-1, 1, c.lv.gid.shape)
+            rf[(4,) + at] = 0.0
+            ref_r = o.restrict(c.lv, lc, rf)
+            rf[(4,) + at] = spike
+            c.se.se_pmg_restrict(P, 0, c.to_gpu(rf), rc)
+            got_r = rc.cpu().numpy().reshape(lc.gid.shape)
+            node = lc.gid[(4,) + tuple(pc // 2 if q else 0 for q in at)]
+            others = lc.gid != node
+            assert np.max(np.abs(got_r - ref_r)[others]) <= 1e-13 * np.max(np.abs(ref_r[others]))
+        c.se.se_pmg_destroy(P)
+    finally:
+        c.close()
+
+
+@pytest.mark.parametrize("pf,pc", PAIRS)
+@pytest.mark.parametrize("value", [np.inf, np.nan, 1e-300, 1e-310])
+def test_transfers_elements_do_not_share_a_fallback(pf, pc, value):
+    c = Case((6, 2, 2), pf, seed=25, bc=("N",) * 6)
+    try:
+        P, lc = _transfer(c, pf, pc)
+        rng = np.random.default_rng(pc)
+        ec, rf = rng.uniform(-1, 1, lc.gid.shape), rng.uniform(-1, 1, c.lv.gid.shape)
+        out = []
+        for put in (False, True):
+            if put:
+                for a in (ec, rf):
+                    a[8] *= 0.0 if abs(value) < 1.0 else 1.0
+                    a[8, 0, 1, 0] = value
+            ef, rc = c.empty(), c.empty(lc.gid.size)
+            c.se.se_pmg_prolong(P, 0, c.to_gpu(ec), ef)
+            c.se.se_pmg_restrict(P, 0, c.to_gpu(rf), rc)
+            out.append((c.to_np(ef), rc.cpu().numpy().reshape(lc.gid.shape)))
+        others = np.arange(c.lv.E) != 8
+        assert np.array_equal(out[0][0][others], out[1][0][others])
+        # the restriction adds the element's results to its neighbours' copies
+        apart = ~np.isin(lc.gid, lc.gid[8])
+        assert np.array_equal(out[0][1][apart], out[1][1][apart])
+        if abs(value) < 1.0:
+            with np.errstate(under="ignore"):
+                ref = o.prolong(c.lv, lc, ec)[8]
+            assert np.max(np.abs(out[1][0][8] - ref)) <= 1e-13 * np.max(np.abs(ref)) + 2e-323 * 8
+        c.se.se_pmg_destroy(P)
+    finally:
+        c.close()
+
+
+@pytest.mark.parametrize("pf,pc", [(2, 1), (5, 3), (8, 4), (10, 9)])
+@pytest.mark.parametrize("k", [-953, -952, -940, 996])
+def test_transfers_of_cancelling_lines_at_the_ends_of_the_range(pf, pc, k):
+    """Odd fields, whose contractions cancel, scaled to the ends of the range of the lines' scale."""
+    c = Case((3, 2, 2), pf, seed=26, bc=("N",) * 6)
+    try:
+        P, lc = _transfer(c, pf, pc)
+        def odd(lv, seed):
+            v = np.random.default_rng(seed).uniform(0.5, 1, lv.gid.shape)
+            v = v - v[:, :, :, ::-1] + 1e-9 * (v[:, :, ::-1] - v)
+            return v / np.max(np.abs(v))
+        ec, rf = odd(lc, 1), odd(c.lv, 2)
+        ef, rc = c.empty(), c.empty(lc.gid.size)
+        c.se.se_pmg_prolong(P, 0, c.to_gpu(np.ldexp(ec, k)), ef)
+        c.se.se_pmg_restrict(P, 0, c.to_gpu(np.ldexp(rf, k)), rc)
+        re, rr = o.prolong(c.lv, lc, ec), o.restrict(c.lv, lc, rf)
+        assert np.max(np.abs(np.ldexp(c.to_np(ef), -k) - re)) <= 1e-13 * np.max(np.abs(re))
+        assert np.max(np.abs(np.ldexp(rc.cpu().numpy().reshape(rr.shape), -k) - rr)) <= 1e-13 * np.max(np.abs(rr))
+        c.se.se_pmg_destroy(P)
+    finally:
+        c.close()
