@@ -9,22 +9,28 @@
 // phase, gathered while its results are produced, gives the shift by which the next phase's
 // readers renormalise to 58 bits, so no phase loses headroom.  The z lines (forward, D^-1, and
 // backward) belong to one thread: their intermediate values stay in registers, D^-1 is applied in
-// FP64 on the line's own scale, and the lines meet again on a common scale after the backward z
-// contraction.  Results leave as doubles, 1/multiplicity taken from the exponent.
+// FP64, and the lines meet again on a common scale after the backward z contraction.  Lines whose
+// results become doubles (forward z, backward x) are read on their own scale: their leading bits cost
+// two instructions per value and no shift back.  Results leave as doubles, 1/multiplicity taken from
+// the exponent.
 //
 // Measured on GB300 (us per launch; in brackets the FP64 kernel this one replaced, at 91% of the FP64
-// pipe): 24^3 elements p = 7 406 [1190], p = 5 168 [460], p = 3 61 [150]; 16^3 p = 9 255 [700].  The
+// pipe): 24^3 elements p = 7 400 [1190], p = 5 166 [460], p = 3 61 [150]; 16^3 p = 9 248 [700].  The
 // multiply-adds keep their pipe (32 lanes/clk/SM) 67% busy; a result's two sums in a row beat all results' sums
 // input by input (more chains in flight, 500 instead of 406 at p = 7: the accumulator stays in the
 // pipe), and 64 registers beat 80 and 96 (440).
 //
-// Error against extended precision (2-norm), over that of the FP64 solve with the same S: 0.36 to 0.45
-// for random and for smooth residuals, 0.5 to 1.6 where the residual decays by eight decades across the
-// window.  58-bit values, both-sign low limbs of S and rounded middle sums matter: with 57 bits and
+// Error against extended precision (2-norm, host emulation, p = 7 / 8 / 10), over that of the FP64 solve
+// with the same S: 0.36 / 0.40 / 0.59 for random and 0.42 / 0.49 / 0.62 for smooth residuals, which is
+// what the kernel is held to.  FP64 keeps the products of S's small entries in full, this kernel on
+// the scale of S's largest entry and of the window: where the residual decays by eight decades from
+// corner to corner of the window 0.56 / 0.92 / 1.07, around one value 10^8 times the others 0.88 / 1.09 /
+// 1.46; the pointwise error there, relative to each value, is 1.2 to 2.6 times FP64's in the geometric
+// mean.  58-bit values, low limbs of S with both signs and rounded middle sums matter: with 57 bits and
 // unsigned limbs the dropped products had a bias and the error was 3 to 5 times FP64's.
 //
-// A block whose values cannot share a scale (infinities, NaN, magnitudes at the ends of the range)
-// computes its elements in FP64 (fdm_slow_block).
+// An element whose values cannot share a scale (infinities, NaN, magnitudes at the ends of the range) is
+// solved in FP64 (fdm_slow_block); the others of its block keep their bits.
 #include <climits>
 
 #include "fdm_window.h"
@@ -40,7 +46,7 @@ struct FdmFxDims {
   static constexpr int VOL = (RS * PB * PB + 1) / 2 * 2;    // 16-byte multiple
   static constexpr int PBP = (PB + 1) / 2 * 2;              // padded matrix row (16-byte loads of two entries)
   static constexpr int SMAT = PB * PBP;                     // one matrix
-  static constexpr int META = 36;                           // magnitudes, exponents and neighbours (ints)
+  static constexpr int META = 36;                           // magnitudes, exponents, fallback, neighbours (ints)
   static constexpr size_t BYTES = (VOL + 6 * SMAT) * 8 + META * 4;
 };
 
@@ -102,17 +108,21 @@ __device__ __forceinline__ double fx_double_any(long long R, int eb) {
 // 2^-log2(multiplicity) of a local point.
 __device__ __forceinline__ int fdm_mult_log2(const uint8_t* pflag, int64_t li) { return __ffs(pflag[li] & 0x0F) - 1; }
 
-// The solve in FP64 (a block with unrepresentable values).  Every thread of the block calls it.
+constexpr int FDM_SLOW = 7;  // index, among an element's ints, of the mark of one without a scale
+
+// The solve in FP64 of the block's marked elements.  Every thread of the block calls it.
 template <int P, int MODE>
-__device__ __noinline__ void fdm_slow_block(const FdmFxArgs& a, int ne, int64_t e0, double* W0, const int* nb0,
+__device__ __noinline__ void fdm_slow_block(const FdmFxArgs& a, int ne, int64_t e0, double* W0, const int* I0,
                                             size_t stride) {
   constexpr int N = P + 1, PB = P + 3, PB2 = PB * PB, PB3 = PB2 * PB;
   constexpr int C0 = MODE == FDM_RAS ? 1 : 0, NC = MODE == FDM_RAS ? N : PB;
   using Dm = FdmFxDims<PB>;
   const int tid = threadIdx.x, le = tid / PB2, ql = tid - le * PB2, p = ql % PB, q = ql / PB;
-  const bool on = le < ne;
-  double* W = reinterpret_cast<double*>(reinterpret_cast<char*>(W0) + (on ? le : 0) * stride);
-  const int* nb = reinterpret_cast<const int*>(reinterpret_cast<const char*>(nb0) + (on ? le : 0) * stride);
+  const int es = le < ne ? le : 0;
+  double* W = reinterpret_cast<double*>(reinterpret_cast<char*>(W0) + es * stride);
+  const int* I = reinterpret_cast<const int*>(reinterpret_cast<const char*>(I0) + es * stride);
+  const int* nb = I + 8;
+  const bool on = le < ne && I[FDM_SLOW] != 0;
   const int64_t e = e0 + le;
   __syncthreads();
   if (on) {
@@ -182,7 +192,7 @@ __global__ void __maxnreg__(fdm_fx_regs<P>()) fdm_fx_kernel(const __grid_constan
   auto W_of = [&](int le) { return reinterpret_cast<double*>(base_of(le)); };
   auto M_of = [&](int le) { return reinterpret_cast<int2*>(base_of(le)) + Dm::VOL; };  // S^T x 3, S x 3
   // ints: [0..2] largest high words (fx_mag) of S_x, S_y, S_z, [3] of the window, [4] of phase x,
-  // [5] phase y, [6] exponent after z, [7] phase y', [8..34] neighbours
+  // [5] phase y, [6] exponent after z, [7] without a scale (FDM_SLOW), [8..34] neighbours
   auto I_of = [&](int le) { return reinterpret_cast<int*>(M_of(le) + 6 * Dm::SMAT); };
   for (int q = tid; q < ne * 8; q += blockDim.x) I_of(q >> 3)[q & 7] = (q & 7) == 6 ? INT_MIN : 0;
   for (int q = tid; q < ne * 27; q += blockDim.x) I_of(q / 27)[8 + q % 27] = a.nbr[27 * e0 + q];
@@ -203,6 +213,16 @@ __global__ void __maxnreg__(fdm_fx_regs<P>()) fdm_fx_kernel(const __grid_constan
 #pragma unroll
   for (int d = 0; d < 3; ++d) s3[d] = on ? a.S[(3 * e + d) * PB2 + ql] : 0.0;
   __syncthreads();
+  // shift that brings a line of results to 63 bits
+  auto line_norm = [](const long long* w, int st) {
+    unsigned high = 0u;
+#pragma unroll
+    for (int q = 0; q < PB; ++q) {
+      const int x = reinterpret_cast<const int*>(w + st * q)[1];
+      high |= (unsigned)(x ^ (x >> 31));
+    }
+    return fx_norm(high);
+  };
   // ---- gather the window (thread: (a, b), loop over c), the matrices' largest entries
   if (on) {
 #pragma unroll
@@ -221,13 +241,18 @@ __global__ void __maxnreg__(fdm_fx_regs<P>()) fdm_fx_kernel(const __grid_constan
   }
   __syncthreads();
   double v[PB];
-  bool bad = false;
+  bool bad = false;   // of the thread's element: S or the window without a scale
+  unsigned low = 0u;  // low words of a line whose high words are all 0
   {
     unsigned m = 0u;
 #pragma unroll
     for (int q = 0; q < PB; ++q) {
       v[q] = W[RS * lp + PS * lq + q];
       m = max(m, fx_mag(v[q]));
+    }
+    if (m == 0u) {
+#pragma unroll 1
+      for (int q = 0; q < PB; ++q) low |= (unsigned)__double2loint(W[RS * lp + PS * lq + q]);
     }
     if (on) {
       fx_group_max(peers, m, mag + 3);
@@ -247,7 +272,8 @@ __global__ void __maxnreg__(fdm_fx_regs<P>()) fdm_fx_kernel(const __grid_constan
     }
   }
   __syncthreads();
-  bad |= fx_bad(mag[3]);
+  bad |= fx_bad(mag[3]) || (mag[3] == 0u && low != 0u);
+  if (on && bad) I[FDM_SLOW] = 1;
   int E = fx_exponent(mag[3]);  // x in units of 2^(E - 1023 - 57)
   auto kS = [&](int d) { return 1079 - fx_exponent(mag[d]); };
   int h[PB], l[PB];
@@ -265,11 +291,7 @@ __global__ void __maxnreg__(fdm_fx_regs<P>()) fdm_fx_kernel(const __grid_constan
     fx_group_max(peers, m, mag + 4);
   }
   E -= kS(0);
-  bad = __syncthreads_or(bad);
-  if (bad) {
-    fdm_slow_block<P, MODE>(a, ne, e0, W_of(0), I_of(0) + 8, Dm::BYTES);
-    return;
-  }
+  bool slow = __syncthreads_or(on && bad);  // some element of the block
   // ---- S_y^T along b (line (alpha, c))
   {
     const int n = fx_norm(mag[4]);
@@ -291,7 +313,7 @@ __global__ void __maxnreg__(fdm_fx_regs<P>()) fdm_fx_kernel(const __grid_constan
   __syncthreads();
   // ---- S_z^T along c, D^-1, S_z (line (alpha, beta)); the line's own scale
   {
-    const int n = fx_norm(mag[5]);
+    const int n = line_norm(WR + lp + RS * lq, PS);
     E += 61 - n;
     long long r3[NC];
     int sft = 0, nl = 0;
@@ -307,7 +329,7 @@ __global__ void __maxnreg__(fdm_fx_regs<P>()) fdm_fx_kernel(const __grid_constan
         v[o] = fx_double_any(fx_dot_row<PB>(ST + 2 * Dm::SMAT + o * PBP, h, l), E - 1 - kS(2)) * dv[o];
         m = max(m, fx_mag(v[o]));
       }
-      bad = fx_bad(m);
+      if (fx_bad(m)) I[FDM_SLOW] = 1;
       const int E2 = fx_exponent(m);
 #pragma unroll
       for (int q = 0; q < PB; ++q) fx_split<58>(v[q], E2, h[q], l[q]);
@@ -323,11 +345,7 @@ __global__ void __maxnreg__(fdm_fx_regs<P>()) fdm_fx_kernel(const __grid_constan
       sft = E2 - 1 - kS(2);
       if (high | any) atomicMax(I + 6, 62 - nl + sft);
     }
-    bad = __syncthreads_or(bad);
-    if (bad) {
-      fdm_slow_block<P, MODE>(a, ne, e0, W_of(0), I_of(0) + 8, Dm::BYTES);
-      return;
-    }
+    slow |= __syncthreads_or(on && I[FDM_SLOW] != 0);
     E = I[6] == INT_MIN ? FX_EMIN : I[6];
     if (on) {
       // x = r3 2^(sft - E + 57): left to 63 bits, then right
@@ -346,7 +364,6 @@ __global__ void __maxnreg__(fdm_fx_regs<P>()) fdm_fx_kernel(const __grid_constan
     const int le2 = tid / (PB * NC), q2 = tid - le2 * PB * NC;
     const bool on2 = le2 < ne;
     const int e2 = on2 ? le2 : 0;
-    const unsigned peers2 = __match_any_sync(__activemask(), on2 ? le2 : -1);
     const int al = q2 % PB, c = C0 + q2 / PB;
     if (on2) {
       const int2* Wl = reinterpret_cast<const int2*>(W_of(e2));
@@ -357,27 +374,22 @@ __global__ void __maxnreg__(fdm_fx_regs<P>()) fdm_fx_kernel(const __grid_constan
         h[q] = x.x;
         l[q] = x.y;
       }
-      unsigned m = 0u;
 #pragma unroll
-      for (int o = 0; o < NC; ++o) {
-        const long long r = fx_dot_row<PB>(Sy + (C0 + o) * PBP, h, l);
-        reinterpret_cast<long long*>(W_of(e2))[al + RS * (C0 + o) + PS * c] = r;
-        m = max(m, fx_high(r));
-      }
-      fx_group_max(peers2, m, reinterpret_cast<unsigned*>(I_of(e2)) + 7);
+      for (int o = 0; o < NC; ++o)
+        reinterpret_cast<long long*>(W_of(e2))[al + RS * (C0 + o) + PS * c] = fx_dot_row<PB>(Sy + (C0 + o) * PBP, h, l);
     }
   }
   __syncthreads();
   // ---- S_x along alpha (line (b', c'), NC^2 lines per element), write out
-  if (tid < ne * NC * NC) {
-    const int le3 = tid / (NC * NC), q3 = tid - le3 * NC * NC;
+  const int le3 = tid / (NC * NC), q3 = tid - le3 * NC * NC;
+  if (le3 < ne && I_of(le3)[FDM_SLOW] == 0) {
     const int b = C0 + q3 % NC, c = C0 + q3 / NC;
     const int* I3 = I_of(le3);
     const unsigned* mag3 = reinterpret_cast<const unsigned*>(I3);
-    const int n = fx_norm(mag3[7]);
     const int Em = I3[6] == INT_MIN ? FX_EMIN : I3[6];
-    const int eb = Em - (1079 - fx_exponent(mag3[1])) + 60 - n - (1079 - fx_exponent(mag3[0]));
     const long long* Wl = reinterpret_cast<const long long*>(W_of(le3)) + RS * b + PS * c;
+    const int n = line_norm(Wl, 1);
+    const int eb = Em - (1079 - fx_exponent(mag3[1])) + 60 - n - (1079 - fx_exponent(mag3[0]));
     const int2* Sx = M_of(le3) + 3 * Dm::SMAT;
 #pragma unroll
     for (int q = 0; q < PB; ++q) fx_renorm<58>(Wl[q], n, h[q], l[q]);
@@ -393,6 +405,7 @@ __global__ void __maxnreg__(fdm_fx_regs<P>()) fdm_fx_kernel(const __grid_constan
       }
     }
   }
+  if (slow) fdm_slow_block<P, MODE>(a, ne, e0, W_of(0), I_of(0), Dm::BYTES);
 }
 
 template <int P, int MODE>

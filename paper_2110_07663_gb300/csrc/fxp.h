@@ -21,7 +21,7 @@
 // Before the final rounding every error is below 2^-55 of (largest value on the scale) x (largest row
 // sum of M); an FP64 dot product rounds each of its terms to 2^-53 of the running sum.  Exponents outside
 // [FX_EMIN, FX_EMAX] (infinities, NaN, values whose results could leave the normal range) are not
-// representable: kernels test for them and compute such elements in FP64.
+// representable: kernels test for them and compute such lines, or elements, in FP64.
 //
 // The arithmetic also compiles as host code, so that its accuracy can be checked without a GPU.
 #pragma once
@@ -210,7 +210,8 @@ SE_FX unsigned fx_mag(double v) {
 }
 
 // Biased exponent of an element whose largest fx_mag is `mag`, and whether it can be represented
-// (an element of zeros is; one whose largest value is below 2^-1022 x 2^-20 counts as zeros).
+// (one of zeros is; so, by the high word alone, is one whose largest value is below 2^-1042: kernels look
+// at the low words where the largest high word is 0).
 SE_FX int fx_exponent(unsigned mag) {
   const int e = (int)(mag >> 20);
   return e > FX_EMIN ? e : FX_EMIN;

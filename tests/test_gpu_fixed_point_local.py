@@ -183,3 +183,36 @@ def test_transfers_of_cancelling_lines_at_the_ends_of_the_range(pf, pc, k):
         c.se.se_pmg_destroy(P)
     finally:
         c.close()
+
+
+@pytest.mark.parametrize("kind", ["ras", "asm"])
+@pytest.mark.parametrize("p", range(2, 11))
+@pytest.mark.parametrize("value", [np.inf, np.nan, 1e-300, 1e-315])
+def test_schwarz_elements_do_not_share_a_fallback(p, kind, value):
+    """Elements far from a window without a scale keep their bits, whatever the number of elements per
+    block; the windows without one do not depend on it either."""
+    c = Case((8, 2, 2), p, seed=27)
+    se = c.se
+    try:
+        sched = (p, 1) if p < 4 else (p, p // 2, 1)
+        P = se.se_pmg_setup(c.m, se.pmg_desc(sched, se.SE_SMOOTH_RAS if kind == "ras" else se.SE_SMOOTH_ASM, 1))
+        r = c.random_continuous(p)
+        g = np.zeros(c.lv.n_global)
+        g[c.lv.gid] = r
+        if abs(value) < 1.0:  # alone in its window and in those beside it
+            g[np.unique(c.lv.gid[[e for e in range(c.lv.E) if e % 8 <= 2]])] = 0.0
+        g[c.lv.gid[1, p // 2, p // 2, p // 2]] = value
+        bad = g[c.lv.gid]
+        s, t, w = c.empty(), c.empty(), c.empty()
+        se.se_pmg_smooth(P, 0, c.to_gpu(r), s)
+        se.se_pmg_smooth(P, 0, c.to_gpu(bad), t)
+        far = np.array([e % 8 >= (5 if abs(value) < 1.0 else 4) for e in range(c.lv.E)])
+        assert np.array_equal(c.to_np(s)[far], c.to_np(t)[far])
+        for ne in (1, 2, 3, 4):
+            se.se_tune_set(p, se.SE_FP64, 0, ne)
+            se.se_pmg_smooth(P, 0, c.to_gpu(bad), w)
+            assert np.array_equal(c.to_np(t), c.to_np(w), equal_nan=True)
+        se.se_pmg_destroy(P)
+    finally:
+        se.se_tune_set(p, se.SE_FP64, 0, 0)
+        c.close()
