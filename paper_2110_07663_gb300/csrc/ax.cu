@@ -395,17 +395,24 @@ __global__ void gs_mask_faces(int nx, int ny, int nz, int bits, T* __restrict__ 
   u[e * N3 + i + N * (j + N * k)] = T(0);
 }
 
-// Where one launch wins: a gathered x-face costs a sector per copy, so the sweeps move less data, but
-// they take two launches.  Measured on GB300 (us of se_gs, sweeps / one launch; FP64, back-to-back
-// launches): p = 7, 4^3 8.5 / 5.0, 8^3 9.7 / 6.6, 12^3 (0.9M points) 12.9 / 9.5, 16^3 (2.1M) 19.2 / 19.3,
-// 24^3 52 / 59, 32^3 114 / 133; p = 3, 16^3 (0.26M) 9.6 / 7.0, 24^3 (0.9M) 13.2 / 13.6, 32^3 19.4 / 22.6;
-// p = 1, 32^3 (0.26M) 12.6 / 8.5.  After the folded operator (fix-up and y/z launch against one): p = 7,
-// 4^3 23.0 / 19.8 with the operator, 12^3 41.3 / 38.9; p = 3, 24^3 36.4 / 39.0.
-// In solves the launches are closer together: FP64 14^3 p = 7 (1.4M) 12.44 ms either way, 20^3 (4.1M)
-// 17.55 / 18.15.  FP32 (half the bytes; us of the FP32 operator): 12^3 p = 9 (1.7M) 52.8 / 48.9, 20^3 p = 7
-// (4.1M) 101.3 / 95.7; solve 14^3 p = 7 5.72 / 5.41 ms.
+// Where one launch wins: its threads are the points on the elements' upper faces, E (3 N^2 - 3 N + 1), and
+// a gathered x-face costs a sector per copy, so the sweeps move less data, but they take two launches
+// (after the folded operator a small fix-up and the y/z launch, which costs less).  Measured on GB300
+// (us, sweeps / one launch, back-to-back calls; M face points).  se_gs FP64: p = 2, 32^3 (0.62M) 14.4 /
+// 12.5, 40^3 (1.22M) 19.7 / 20.7; p = 3, 20^3 (0.30M) 11.4 / 8.3, 24^3 (0.51M) 12.4 / 12.4, 28^3 (0.81M)
+// 15.0 / 16.4; p = 5, 20^3 (0.73M) 16.5 / 14.4; p = 7, 12^3 (0.29M) 12.4 / 8.3, 16^3 (0.69M) 14.4 / 14.4, 20^3
+// (1.35M) 20.7 / 22.6; p = 9, 14^3 (0.74M) 16.5 / 14.4; p = 1, 48^3 (0.77M) 19.0 / 14.5, 64^3 (1.84M) 32.9 /
+// 28.8.  The folded operator with its QQ^T: p = 3, 18^3 (0.22M) 26.7 / 24.7, 20^3 (0.30M) 32.1 / 32.0, 24^3
+// (0.51M) 35.0 / 37.0; p = 5, 16^3 (0.37M) 37.8 / 38.0; p = 7, 12^3 39.0 / 37.0, 13^3 (0.37M) 45.3 / 45.1, 16^3 79.7 /
+// 81.8; p = 9, 11^3 (0.36M) 67.7 / 67.7.  The FP32 operator with its QQ^T: p = 3, 24^3 31.6 / 29.6, 32^3 (1.21M)
+// 52.5 / 51.8; p = 7, 20^3 102.1 / 97.9; p = 1, 64^3 57.9 / 51.7.
 template <typename T>
-static bool gs_one_launch(const Level& lv) { return lv.L <= (sizeof(T) == 4 ? 5000000 : 1300000); }
+static bool gs_one_launch(const Level& lv, bool folded) {
+  const int64_t points = lv.E * (3 * lv.N * lv.N - 3 * lv.N + 1);
+  if (folded) return points <= 375000;
+  if (lv.N == 2) return points <= 1900000;
+  return points <= (sizeof(T) == 4 ? 1400000 : 700000);
+}
 
 // QQ^T in one launch: a thread per point on an element's upper faces (i, j or k = p) whose copies the
 // element owns (no lower neighbour shares them) gathers the node's 2, 4 or 8 copies, sums them in the
@@ -528,7 +535,7 @@ static int gs_sweeps(const Level& lv, T* u, bool mask, double bytes, double flop
   if (mask)
     for (int f = 0; f < 6; ++f)
       if (lv.bc[f] == SE_BC_DIRICHLET) bits |= 1 << f;
-  if (gs_one_launch<T>(lv)) return gs_all<T, N>(lv, 0, bits, u, var, bytes, flops, s);
+  if (gs_one_launch<T>(lv, false)) return gs_all<T, N>(lv, 0, bits, u, var, bytes, flops, s);
   if (bits && nx == 1) {  // no x sweep to carry the mask
     {
       const int64_t n = 2 * N2 * ((int64_t)ny * nz + (int64_t)nx * nz + (int64_t)nx * ny);
@@ -589,7 +596,7 @@ static int gs_after_fold(const Level& lv, double* y, int NE, cudaStream_t s) {
   // the x direction must be complete before the y sweep adds across y-interfaces: a copy summed
   // across a block-boundary x-interface after the y sweep would count its y-partner's x-neighbour
   // twice
-  if (gs_one_launch<double>(lv)) {
+  if (gs_one_launch<double>(lv, true)) {
     const double copies = yz_copies<N>(nx, ny, nz);
     return gs_all<double, N>(lv, NE, 0, y, var, 2.0 * copies * sizeof(double), copies / 2, s);
   }
