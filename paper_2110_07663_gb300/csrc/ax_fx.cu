@@ -23,8 +23,8 @@
 // left to gs_fold_fixup_x.
 //
 // Measured on GB300 (us per launch; in brackets the even-odd FP64 kernel this one replaced, which ran at
-// the FP64 pipe's 2 FMA/clk/SM): 32^3 elements p = 7 420 [1420], p = 5 205 [525], p = 3 55 [138]; even
-// orders (unfolded in FP64) 20^3 p = 8 178 [725].  Memory needs 158 us of the 420 and the 9 FP64
+// the FP64 pipe's 2 FMA/clk/SM): 32^3 elements p = 7 414 [1420], p = 5 204 [525], p = 3 54 [138]; even
+// orders (unfolded in FP64) 20^3 p = 8 179 [725].  Memory needs 158 us of the 414 and the 9 FP64
 // instructions per point 240; what bounds it is about 500 instructions per 32 points, 72 of them
 // multiply-adds of 3.5 cycles each, at the 32 warps that its registers and shared memory allow (no
 // pipe is full, each waits for the others in turn).  64 registers beat 48, 56, 72 and more;
@@ -67,16 +67,17 @@ __device__ __forceinline__ bool fx_split_line(const double* p, int st, int (&h)[
     v[q] = p[st * q];
     mag = max(mag, fx_mag(v[q]));
   }
+  bool scaled = !fx_bad(mag);
+  if (mag == 0u) {  // zeros, or values so small that their high words are
+    unsigned low = 0u;
+#pragma unroll
+    for (int q = 0; q < N; ++q) low |= (unsigned)__double2loint(v[q]);
+    scaled = low == 0u;
+  }
   E = fx_exponent(mag);
 #pragma unroll
   for (int q = 0; q < N; ++q) fx_split(v[q], E, h[q], l[q]);
-  if (mag == 0u) {  // zeros, or values so small that their high words are
-    unsigned low = 0u;
-#pragma unroll 1
-    for (int q = 0; q < N; ++q) low |= (unsigned)__double2loint(p[st * q]);
-    return low == 0u;
-  }
-  return !fx_bad(mag);
+  return scaled;
 }
 
 // out = M in along a line without a scale, in FP64: M = D, or D^T.  in and out may be the same line.

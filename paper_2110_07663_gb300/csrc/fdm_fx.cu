@@ -251,8 +251,8 @@ __global__ void __maxnreg__(fdm_fx_regs<P>()) fdm_fx_kernel(const __grid_constan
       m = max(m, fx_mag(v[q]));
     }
     if (m == 0u) {
-#pragma unroll 1
-      for (int q = 0; q < PB; ++q) low |= (unsigned)__double2loint(W[RS * lp + PS * lq + q]);
+#pragma unroll
+      for (int q = 0; q < PB; ++q) low |= (unsigned)__double2loint(v[q]);
     }
     if (on) {
       fx_group_max(peers, m, mag + 3);
