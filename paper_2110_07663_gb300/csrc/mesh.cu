@@ -402,7 +402,6 @@ int se_mesh_create(const se_mesh_desc* desc, se_mesh_t* out) {
   box_lengths(m);
   if ((st = build_level(m, desc->p, &m->fine, m->allocs, m->stream)) != SE_OK) return fail(st);
   if ((st = build_jacobi(m->fine, m->allocs, m->scratch, m->stream)) != SE_OK) return fail(st);
-  if ((st = dmalloc(m->allocs, &m->tmp64, (size_t)m->fine.L)) != SE_OK) return fail(st);
   if ((st = dmalloc(m->allocs, &m->tmpa32, (size_t)m->fine.L)) != SE_OK) return fail(st);
   if ((st = dmalloc(m->allocs, &m->tmpb32, (size_t)m->fine.L)) != SE_OK) return fail(st);
   if (cudaStreamSynchronize(m->stream) != cudaSuccess) {

@@ -173,7 +173,6 @@ struct se_mesh_s {
   cudaStream_t stream = nullptr;
   se::Allocs allocs;
   se::Scratch scratch;
-  double* tmp64 = nullptr;       // [L] work vector
   float* tmpa32 = nullptr;       // [L]
   float* tmpb32 = nullptr;       // [L]
   float* tmpc32 = nullptr;       // [L], allocated by the first FP32 se_residual

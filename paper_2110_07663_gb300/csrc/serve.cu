@@ -47,7 +47,7 @@ size_t footprint_bytes(const se_mesh_desc& d, const se_pmg_desc& pd) {
     // X 24, G 48, B 8, dinv 8 + 4, flags 1, QQ^T ids ~4, vectors 7 in the V-cycle precision
     double per_pt = 24 + 48 + 8 + 12 + 1 + 4 + 7 * vec;
     if (fp32 && l + 1 < pd.nlev) per_pt += 24;                  // FP32 geometric factors
-    if (l == 0) per_pt += 5 * 8 + 8 + 8;                         // Krylov vectors, temporaries
+    if (l == 0) per_pt += 5 * 8 + 8;                             // Krylov vectors, FP32 temporaries
     total += L * per_pt;
     if (l + 1 < pd.nlev && pd.smoother != SE_SMOOTH_JACOBI) {
       const double fdm = 3 * pb * pb * 8 + 3 * pb * 8 + pb * pb * pb * 8 +

@@ -316,7 +316,7 @@ int restrict_apply(const Level& f, const Level& c, const T* J, const T* rf, T* r
                    f.E * (Nf * Nf * Nf * (sizeof(T) + 1.0) + Nc * Nc * Nc * sizeof(T)),
                    2.0 * f.E * (Nf * Nf * Nf * Nc + Nf * Nf * Nc * Nc + Nf * Nc * Nc * Nc),
                    prof_variant<T>(f.p));
-    int st = SE_OK;
+    [[maybe_unused]] int st = SE_OK;
     if constexpr (sizeof(T) == 8) {
       SE_TRY(transfer_fx(f, c, true, J, rf, rc, false, s));
     } else if (transfer_eo<T, true>(f, c, J, rf, f.pflag, rc, false, s, &st)) {
@@ -337,12 +337,15 @@ int prolong_apply(const Level& f, const Level& c, const T* J, const T* ec, T* ef
                  f.E * (Nf * Nf * Nf * (accumulate ? 2.0 : 1.0) + Nc * Nc * Nc) * sizeof(T),
                  2.0 * f.E * (Nc * Nc * Nc * Nf + Nc * Nc * Nf * Nf + Nc * Nf * Nf * Nf),
                  prof_variant<T>(f.p));
-  if constexpr (sizeof(T) == 8) return transfer_fx(f, c, false, J, ec, ef, accumulate, s);
-  int st = SE_OK;
-  if (transfer_eo<T, false>(f, c, J, ec, nullptr, ef, accumulate, s, &st)) return st;
-  transfer_kernel<T, false><<<(unsigned)f.E, 128, 0, s>>>(f.N, c.N, J, ec, nullptr, ef, accumulate);
-  SE_LAUNCH_CHECK();
-  return SE_OK;
+  if constexpr (sizeof(T) == 8) {
+    return transfer_fx(f, c, false, J, ec, ef, accumulate, s);
+  } else {
+    int st = SE_OK;
+    if (transfer_eo<T, false>(f, c, J, ec, nullptr, ef, accumulate, s, &st)) return st;
+    transfer_kernel<T, false><<<(unsigned)f.E, 128, 0, s>>>(f.N, c.N, J, ec, nullptr, ef, accumulate);
+    SE_LAUNCH_CHECK();
+    return SE_OK;
+  }
 }
 
 template int restrict_apply<double>(const Level&, const Level&, const double*, const double*, double*, cudaStream_t);
