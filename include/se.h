@@ -344,8 +344,9 @@ int se_batch_info(se_batch_t batch, int* groups, int* grouped_problems);
  * precision.  se_tune times every valid candidate on a scratch problem of about 2M points
  * (allocating its own buffers), keeps the fastest in the process-wide table used by all later
  * launches, and reports it with the measured per-launch times.  se_tune_get reports the
- * values in use (the built-in heuristic until tuned); se_tune_set installs given values
- * (0 = heuristic). */
+ * values in use (until tuned, those of the built-in heuristic for meshes of many elements; it takes
+ * smaller blocks where few elements would leave multiprocessors idle); se_tune_set installs given
+ * values (0 = heuristic). */
 typedef struct se_tile_cfg {
   int p;
   int precision;              /* SE_FP64 or SE_FP32 */

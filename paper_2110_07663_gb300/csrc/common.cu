@@ -199,19 +199,34 @@ int scratch_alloc(Allocs& a, Scratch* s) {
 static std::mutex g_tile_mu;
 static TileCfg g_tiles[SE_MAX_ORDER + 1][2];
 
-// The busiest of the 152 multiprocessors holds ne ceil(ceil(E / ne) / 152) elements; smaller blocks cost
+// Multiprocessors of the current device, asked once per device.
+static int sm_count() {
+  constexpr int DEVICES = 64;
+  static std::atomic<int> known[DEVICES];
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= DEVICES) return 152;
+  n = known[dev].load(std::memory_order_relaxed);
+  if (n == 0) {
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) n = 152;
+    known[dev].store(n, std::memory_order_relaxed);
+  }
+  return n;
+}
+
+// The busiest of the M multiprocessors holds ne ceil(ceil(E / ne) / M) elements; smaller blocks cost
 // up to a fifth more per element (measured at large E: p = 7 FDM 3 elements 403 us, 2 424, 1 485).
 // Measured on GB300, us per FDM launch with 1 / 2 / 3 elements: p = 7, E = 64 18.7 / 21.1 / 24.8, 216 21.4 /
 // 21.8 / 24.9, 512 31.2 / 29.4 / 36.5, 1000 47.0 / 45.8 / 47.3; p = 9, E = 64 26.9 / 31.1 / 37.1, 512 50.4 /
 // 49.1 / 61.6; operator p = 8, E = 64 16.9 / 20.8 / 22.1, p = 9 19.0 / 22.6.
 int balanced_elems(int64_t E, int most) {
   if (E <= 0) return most;
+  const int sms = sm_count();
   int best = most;
   double least = 0.0;
   for (int ne = most; ne >= 1; --ne) {
     const double f = most > 1 ? (double)(most - ne) / (most - 1) : 0.0;
     const int64_t blocks = (E + ne - 1) / ne;
-    const double cost = (double)(ne * ((blocks + 151) / 152)) * (1.0 + 0.2 * f * f);
+    const double cost = (double)(ne * ((blocks + sms - 1) / sms)) * (1.0 + 0.2 * f * f);
     if (ne == most || cost < least) {
       least = cost;
       best = ne;
