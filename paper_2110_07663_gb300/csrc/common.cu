@@ -218,9 +218,14 @@ static int sm_count() {
 // Measured on GB300, us per FDM launch with 1 / 2 / 3 elements: p = 7, E = 64 18.7 / 21.1 / 24.8, 216 21.4 /
 // 21.8 / 24.9, 512 31.2 / 29.4 / 36.5, 1000 47.0 / 45.8 / 47.3; p = 9, E = 64 26.9 / 31.1 / 37.1, 512 50.4 /
 // 49.1 / 61.6; operator p = 8, E = 64 16.9 / 20.8 / 22.1, p = 9 19.0 / 22.6.
+// From 4 blocks of `most` per multiprocessor several are resident at once and fill each other's tail: `most`
+// is then no worse, and up to a tenth better (this rule / `most`: p = 4, 16^3 FDM 43.1 / 39.3, p = 5, 20^3
+// operator 64.1 / 58.4, p = 6, 16^3 52.6 / 48.9); below, `most` loses (p = 8, 10^3 FDM 58.7 / 62.1, p = 9
+// 78.3 / 85.6, p = 4, 12^3 operator 14.5 / 16.6).
 int balanced_elems(int64_t E, int most) {
   if (E <= 0) return most;
   const int sms = sm_count();
+  if ((E + most - 1) / most > 4 * sms) return most;
   int best = most;
   double least = 0.0;
   for (int ne = most; ne >= 1; --ne) {
