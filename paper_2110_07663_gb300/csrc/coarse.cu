@@ -733,6 +733,12 @@ static int coarse_kernel_attrs() {
   return SE_OK;
 }
 
+// Synchronisation words of a solve: arrival count at 0, status, then the blocks' flags, in one piece (one
+// reset per solve) but on 128-byte lines of their own: every block polls the count while its
+// neighbours' flags are written.  us per iteration with all in one line / on their own: n = 4913 7.0 / 6.8,
+// n = 15625 7.1 / 6.8, n = 35937 7.9 / 7.4; up to n = 2197 within 2% either way.
+constexpr int SYNC_STATUS = 32, SYNC_FLAGS = 64;
+
 // Partial sums of the summing barrier: two buffers of 4 doubles per block.
 size_t coarse_partial_doubles(int nblocks) { return 8 * (size_t)nblocks; }
 
@@ -768,11 +774,10 @@ int coarse_alloc(const Level& lv, Allocs& allocs, CoarseWork* w) {
   for (double** v : {&w->x, &w->r, &w->u, &w->p, &w->q, &w->s, &w->z, &w->w0, &w->w1})
     SE_TRY(dmalloc(allocs, v, n));
   SE_TRY(dmalloc(allocs, &w->partial, coarse_partial_doubles(w->nblocks)));
-  // count, status and flags in one piece: one reset per solve
-  SE_TRY(dmalloc(allocs, &w->bar, 4 + (size_t)w->nblocks));
-  w->status = reinterpret_cast<int*>(w->bar + 2);
-  w->flags = w->bar + 4;
-  SE_TRY(dzero(w->bar, (4 + (size_t)w->nblocks) * sizeof(unsigned), allocs.stream));
+  SE_TRY(dmalloc(allocs, &w->bar, SYNC_FLAGS + (size_t)w->nblocks));
+  w->status = reinterpret_cast<int*>(w->bar + SYNC_STATUS);
+  w->flags = w->bar + SYNC_FLAGS;
+  SE_TRY(dzero(w->bar, (SYNC_FLAGS + (size_t)w->nblocks) * sizeof(unsigned), allocs.stream));
   SE_TRY(dmalloc(allocs, &w->totals, 3));
   SE_TRY(dzero(w->totals, 3 * sizeof(unsigned long long), allocs.stream));
   return SE_OK;
@@ -812,8 +817,8 @@ int coarse_solve(const Level& lv, CoarseWork& w, const T* r_l, T* x_l, double to
   a.timeout_ns = BARRIER_TIMEOUT_NS;
   ProfScope prof(SE_K_COARSE, s, (double)lv.n_global, 0.0, 0.0);
   const bool reg = w.flags && lv.n_global <= (int64_t)w.nblocks * CG_THREADS;
-  // bar[2], status[2] and the flags are contiguous (coarse_alloc, the static work space)
-  SE_CUDA(cudaMemsetAsync(w.bar, 0, (4 + (reg ? (size_t)w.nblocks : 0)) * sizeof(unsigned), s));
+  // count, status and flags are one piece (coarse_alloc, the static work space)
+  SE_CUDA(cudaMemsetAsync(w.bar, 0, (SYNC_FLAGS + (reg ? (size_t)w.nblocks : 0)) * sizeof(unsigned), s));
   void* args[] = {&a};
   SE_TRY(coarse_kernel_attrs());
   SE_CUDA(cudaLaunchCooperativeKernel(reg ? (const void*)coarse_reg_kernel<T> : (const void*)coarse_pcg_kernel<T>,
@@ -1008,16 +1013,15 @@ extern "C" int se_selftest_wait_timeout(double timeout_ms) {
 // ------------------------------------------------------------------ coarse solve, no allocation
 // Scratch of se_pmg_coarse_solve_noalloc: the nine pipelined-CG vectors (x, r, u, p, q, s, z and
 // the two alternating w) of at most NOALLOC_MAX_N coarse nodes, the per-block partial sums
-// (two buffers of 4 doubles per block), and four 32-bit words at the end (barrier count and an
-// unused word, status, iteration count).  It lives in the library's static device memory: every
+// (two buffers of 4 doubles per block), and the synchronisation words (SYNC_FLAGS words and a flag
+// per block).  It lives in the library's static device memory: every
 // GPU that loads the library holds it until the process exits.
 namespace se {
 constexpr int64_t NOALLOC_MAX_N = 1 << 17;        // 131072 coarse (p = 1) global nodes
 constexpr int NOALLOC_MAX_BLOCKS = 1024;
 constexpr int NOALLOC_VECTORS = 9;
-// vectors, partial sums, barrier and status words, per-block flags
-constexpr int64_t NOALLOC_WORDS =
-    NOALLOC_VECTORS * NOALLOC_MAX_N + 8 * NOALLOC_MAX_BLOCKS + 2 + NOALLOC_MAX_BLOCKS / 2;
+constexpr int64_t NOALLOC_WORDS = NOALLOC_VECTORS * NOALLOC_MAX_N + 8 * NOALLOC_MAX_BLOCKS +
+                                  (SYNC_FLAGS + NOALLOC_MAX_BLOCKS) / 2;
 static __device__ __align__(256) double g_coarse_scratch[NOALLOC_WORDS];
 
 // Host code must not use g_coarse_scratch itself (that name is a host-side stand-in): the
@@ -1050,8 +1054,8 @@ extern "C" int se_pmg_coarse_solve_noalloc(se_pmg_t P, const double* r, double* 
   for (int k = 0; k < NOALLOC_VECTORS; ++k) *vecs[k] = base + k * NOALLOC_MAX_N;
   w.partial = base + NOALLOC_VECTORS * NOALLOC_MAX_N;  // coarse_partial_doubles(nblocks) <= 8 * 1024
   w.bar = reinterpret_cast<unsigned*>(base + NOALLOC_VECTORS * NOALLOC_MAX_N + 8 * NOALLOC_MAX_BLOCKS);
-  w.status = reinterpret_cast<int*>(w.bar + 2);
-  w.flags = reinterpret_cast<unsigned*>(base + NOALLOC_VECTORS * NOALLOC_MAX_N + 8 * NOALLOC_MAX_BLOCKS + 2);
+  w.status = reinterpret_cast<int*>(w.bar + SYNC_STATUS);
+  w.flags = w.bar + SYNC_FLAGS;
   // coarse_solve zeroes the barrier, status and flag words before its launch; the vectors are fully
   // written before they are read
   SE_TRY(coarse_solve<double>(c, w, r, x, P->desc.coarse_tol, P->desc.coarse_maxit, s));
