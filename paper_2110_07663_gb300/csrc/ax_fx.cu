@@ -25,17 +25,17 @@
 // Measured on GB300 (us per launch; in brackets the even-odd FP64 kernel this one replaced, which ran at
 // the FP64 pipe's 2 FMA/clk/SM): 32^3 elements p = 7 414 [1420], p = 5 204 [525], p = 3 54 [138]; even
 // orders (unfolded in FP64) 20^3 p = 8 179 [725].  Memory needs 158 us of the 414 and the 9 FP64
-// instructions per point 240; what bounds it is about 500 instructions per 32 points, 72 of them
+// instructions per point 240; what bounds it is about 498 instructions per 32 points, 72 of them
 // multiply-adds of 3.5 cycles each, at the 32 warps that its registers and shared memory allow (no
 // pipe is full, each waits for the others in turn).  64 registers beat 48, 56, 72 and more;
 // prefetching G to L2 costs more instructions than it saves waits.  w on one scale per element was 2%
 // faster at p = 7 (406), but a small value then lost the bits below 2^-56 of the element's largest one,
 // though no line joins them; the parts of y as doubles, added in FP64, cost about 470.
 //
-// Error against extended precision (2-norm, host emulation on perturbed meshes, p = 2 to 10), over that
-// of the FP64 dot products: 0.37 to 0.78 for random values, 0.39 to 0.50 for smooth ones, 0.31 to
-// 0.56 for values that decay by eight decades across the element, 0.29 to 0.74 around one value 10^8
-// times the others; away from that value's lines the points keep FP64's accuracy.
+// Error against extended precision (2-norm, host emulation on plain and perturbed meshes, p = 2, 3, 7, 8
+// and 10), over that of the FP64 dot products: 0.40 to 0.78 for random values, 0.40 to 0.50 for smooth
+// ones, 0.32 to 0.67 for values that decay by eight decades across the element, 0.29 to 0.74 around one
+// value 10^8 times the others; away from that value's lines the points keep FP64's accuracy.
 //
 // A line whose values cannot share a scale (infinities, NaN, magnitudes at the ends of the range) is
 // contracted in FP64 (ax_slow_line); what does not touch it keeps its bits.
