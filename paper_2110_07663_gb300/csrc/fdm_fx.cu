@@ -15,19 +15,20 @@
 // the exponent.
 //
 // Measured on GB300 (us per launch; in brackets the FP64 kernel this one replaced, at 91% of the FP64
-// pipe): 24^3 elements p = 7 400 [1190], p = 5 166 [460], p = 3 61 [150]; 16^3 p = 9 248 [700].  The
-// multiply-adds keep their pipe (32 lanes/clk/SM) 65% busy; a result's two sums in a row beat all results' sums
+// pipe): 24^3 elements p = 7 377 [1190], p = 5 158 [460], p = 3 59 [150]; 16^3 p = 9 236 [700].  The
+// multiply-adds keep their pipe (32 lanes/clk/SM) about 68% busy; a result's two sums in a row beat all results' sums
 // input by input (more chains in flight, 500 instead of 406 at p = 7: the accumulator stays in the
 // pipe), and 64 registers beat 80 and 96 (440).
 //
-// Error against extended precision (2-norm, host emulation, p = 7 / 8 / 10), over that of the FP64 solve
-// with the same S: 0.36 / 0.40 / 0.59 for random and 0.42 / 0.49 / 0.62 for smooth residuals, which is
-// what the kernel is held to.  FP64 keeps the products of S's small entries in full, this kernel on
-// the scale of S's largest entry and of the window: where the residual decays by eight decades from
-// corner to corner of the window 0.56 / 0.92 / 1.07, around one value 10^8 times the others 0.88 / 1.09 /
-// 1.46; the pointwise error there, relative to each value, is 1.2 to 2.6 times FP64's in the geometric
-// mean.  58-bit values, low limbs of S with both signs and rounded middle sums matter: with 57 bits and
-// unsigned limbs the dropped products had a bias and the error was 3 to 5 times FP64's.
+// Error against extended precision (2-norm, host emulation, p = 2 to 10), over that of the FP64 solve with
+// the same S: 0.31 to 0.43 for random and 0.33 to 0.44 for smooth residuals, 0.34 to 0.70 where the
+// residual decays by eight decades across the window, 0.41 to 0.99 around one value 10^8 times the
+// others.  FP64 keeps the products of S's small entries in full, this kernel on the scale of S's
+// largest entry and of the window, so the error relative to each value by itself is up to 1.5 and 1.8
+// times FP64's (geometric mean) in the last two.  58-bit values, low limbs with both signs, in S and in
+// the values, and rounded middle sums matter: with 57 bits and unsigned limbs the dropped products had a
+// bias and the error was 3 to 5 times FP64's; with unsigned limbs of the values it was up to 1.5
+// times around a large value, and the masks cost 24 us at p = 7 (400).
 //
 // An element whose values cannot share a scale (infinities, NaN, magnitudes at the ends of the range) is
 // solved in FP64 (fdm_slow_block); the others of its block keep their bits.
@@ -262,10 +263,7 @@ __global__ void __maxnreg__(fdm_fx_regs<P>()) fdm_fx_kernel(const __grid_constan
         const unsigned ms = mag[d];
         bad |= fx_bad(ms);
         int h, l;
-        fx_split(s3[d], fx_exponent(ms), h, l);
-        const int up = (l + (int)FX_HALF) >> FX_LIMB;  // |low limb| <= 2^27 (larger dropped products otherwise)
-        h += up;
-        l -= up << FX_LIMB;
+        fx_split<57, true>(s3[d], fx_exponent(ms), h, l);
         SR[d * Dm::SMAT + lq * PBP + lp] = make_int2(h, l);
         ST[d * Dm::SMAT + lp * PBP + lq] = make_int2(h, l);
       }
@@ -348,13 +346,13 @@ __global__ void __maxnreg__(fdm_fx_regs<P>()) fdm_fx_kernel(const __grid_constan
     slow |= __syncthreads_or(on && I[FDM_SLOW] != 0);
     E = I[6] == INT_MIN ? FX_EMIN : I[6];
     if (on) {
-      // x = r3 2^(sft - E + 57): left to 63 bits, then right
+      // x = r3 2^(sft - E + 57): left to 63 bits, then right (by 5 at least)
       const int right = nl - (sft - E + 57);
 #pragma unroll
       for (int o = 0; o < NC; ++o) {
-        const long long x = fx_shr((long long)((unsigned long long)r3[o] << nl), right);
-        reinterpret_cast<int2*>(W)[lp + RS * lq + PS * (C0 + o)] =
-            make_int2((int)(x >> FX_LIMB), (int)((unsigned)x & 0x0fffffffu));
+        int xh, xl;
+        fx_shift_limbs((long long)((unsigned long long)r3[o] << nl), right - 1, xh, xl);
+        reinterpret_cast<int2*>(W)[lp + RS * lq + PS * (C0 + o)] = make_int2(xh, xl);
       }
     }
   }

@@ -221,8 +221,10 @@ SE_FX bool fx_bad(unsigned mag) {
 }
 
 // v in units of 2^(E - 1023 - (XB - 1)), |x| < 2^XB, E >= every value's biased exponent.  XB = 57, or
-// 58 where lines are not folded (a folded sum needs the bit).
-template <int XB = 57>
+// 58 where lines are not folded (a folded sum needs the bit).  NEAR: |l| <= 2^27 of either sign, which
+// halves the low x low products that a contraction leaves out, for one more operation; a folded sum of
+// two low limbs needs their sign to be the value's.
+template <int XB = 57, bool NEAR = XB == 58>
 SE_FX void fx_split(double v, int E, int& h, int& l) {
   unsigned hi, lo;
   fx_words(v, hi, lo);
@@ -234,8 +236,14 @@ SE_FX void fx_split(double v, int E, int& h, int& l) {
   const unsigned top = (fx_funnel_l(lo, hi, UP) & (one - 1u)) | one;
   const unsigned long long x = fx_shr(((unsigned long long)top << 32) | (lo << UP), sh);
   // both limbs take the sign: a zero, or a value shifted out, has two zero limbs whatever its sign
-  h = ((int)(unsigned)(x >> 32) ^ s) - s;
-  l = ((int)((unsigned)x >> 4) ^ s) - s;
+  const unsigned xl = (unsigned)x;
+  if constexpr (NEAR) {
+    h = ((int)((unsigned)(x >> 32) + (xl >> 31)) ^ s) - s;
+    l = (((int)xl >> 4) ^ s) - s;
+  } else {
+    h = ((int)(unsigned)(x >> 32) ^ s) - s;
+    l = ((int)(xl >> 4) ^ s) - s;
+  }
 }
 
 // The double nearest to R 2^(eb - 1023), |R| < 2^63; eb >= 1 and eb + 63 < 2046 (callers bound
@@ -270,14 +278,23 @@ SE_FX unsigned fx_high(long long R) {
 // Left shift that brings values whose largest high word is `high` to 63 bits.
 SE_FX int fx_norm(unsigned high) { return high ? 30 - fx_bfind(high) : 30; }
 
-// Limbs of R after a left shift by n to 63 bits: x = R 2^n / 2^(63 - XB), |x| < 2^XB.
+// Limbs of R after a left shift by n to 63 bits: x = R 2^n / 2^(63 - XB), |x| < 2^XB, |l| <= 2^27.
 template <int XB = 57>
 SE_FX void fx_renorm(long long R, int n, int& h, int& l) {
   const unsigned long long x = (unsigned long long)R << n;
   const int xh = (int)(x >> 32);
-  constexpr int DOWN = 63 - XB;
-  h = xh >> (DOWN + FX_LIMB - 32);
-  l = (int)(fx_funnel_r((unsigned)x, (unsigned)xh, DOWN) & 0x0fffffffu);
+  constexpr int UP = 63 - XB + FX_LIMB - 32;  // bits of x's high word below h
+  const unsigned w = fx_funnel_r((unsigned)x, (unsigned)xh, UP);  // l, and bits below it, at the top
+  h = (xh >> UP) + (int)(w >> 31);
+  l = (int)w >> (32 - FX_LIMB);
+}
+
+// Limbs of x 2^-(s + 1), s >= 0, rounded; |l| <= 2^27.
+SE_FX void fx_shift_limbs(long long x, int s, int& h, int& l) {
+  const long long y = (fx_shr(x, s) + 1) >> 1;
+  const unsigned w = (unsigned)y << (32 - FX_LIMB);
+  h = (int)(y >> FX_LIMB) + (int)(w >> 31);
+  l = (int)w >> (32 - FX_LIMB);
 }
 
 #ifdef __CUDACC__
