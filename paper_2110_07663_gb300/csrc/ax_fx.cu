@@ -23,12 +23,12 @@
 // left to gs_fold_fixup_x.
 //
 // Measured on GB300 (us per launch; in brackets the even-odd FP64 kernel this one replaced, which ran at
-// the FP64 pipe's 2 FMA/clk/SM): 32^3 elements p = 7 414 [1420], p = 5 204 [525], p = 3 54 [138]; even
-// orders (unfolded in FP64) 20^3 p = 8 179 [725].  Memory needs 158 us of the 414 and the 9 FP64
+// the FP64 pipe's 2 FMA/clk/SM): 32^3 elements p = 7 408 [1420], p = 5 203 [525], p = 3 54 [138]; even
+// orders (unfolded in FP64) 20^3 p = 8 179 [725].  Memory needs 158 us of the 408 and the 9 FP64
 // instructions per point 240; what bounds it is about 498 instructions per 32 points, 72 of them
 // multiply-adds of 3.5 cycles each, at the 32 warps that its registers and shared memory allow (no
 // pipe is full, each waits for the others in turn).  64 registers beat 48, 56, 72 and more;
-// prefetching G to L2 costs more instructions than it saves waits.  w on one scale per element was 2%
+// prefetching G to L2 costs more instructions than it saves waits.  w on one scale per element was 0.5%
 // faster at p = 7 (406), but a small value then lost the bits below 2^-56 of the element's largest one,
 // though no line joins them; the parts of y as doubles, added in FP64, cost about 470.
 //
@@ -139,6 +139,42 @@ __device__ __forceinline__ double ax_fx_input(const AxFxArgs& a, int64_t gi, boo
   return zero ? 0.0 : v;
 }
 
+// The three parts of a result, each on its own scale, added on the largest of them (what a smaller one
+// loses there is below 2^-60 of the sum's largest part) and rounded to double once.
+__device__ __forceinline__ double ax_sum(long long t, int et, long long r, int er, long long s, int es, int k) {
+  const int m = max(et, max(er, es));
+  return fx_double(fx_shr(t, m - et) + fx_shr(r, m - er) + fx_shr(s, m - es), m - k);
+}
+
+// The last step of a column (i, j) where the column or a line through it has no scale (in a function of
+// its own, out of the kernel's instruction stream): points without such a line get the same bits as ever.
+template <int N>
+__device__ __noinline__ void ax_slow_column(const double* D, const FxFold<N, N>& tT, double* U, int i, int j) {
+  using Dm = AxFxDims<N>;
+  constexpr int PL = Dm::PLANE;
+  double* u = U + i + Dm::NP * j;
+  int h[N], l[N], E;
+  if (fx_split_line<N>(u, PL, h, l, E)) {
+    fx_contract<N, N, -1>(tT, h, l, [&](int q, long long r) { reinterpret_cast<long long*>(u)[PL * q] = r; });
+  } else {
+    ax_slow_line<N>(D, true, u, u, PL);
+    E = FX_NO_SCALE;
+  }
+  auto value = [&](const double* p, int e) {
+    return e == FX_NO_SCALE ? *p : fx_double(*reinterpret_cast<const long long*>(p), e - tT.k);
+  };
+#pragma unroll 1
+  for (int q = 0; q < N; ++q) {
+    double *t = u + PL * q, *r = t + Dm::VOL, *s = r + Dm::VOL;
+    const int er = *ax_line_scale<N>(U, 1, j, q), es = *ax_line_scale<N>(U, 2, i, q);
+    if (max(E, max(er, es)) != FX_NO_SCALE)
+      *t = ax_sum(*reinterpret_cast<const long long*>(t), E, *reinterpret_cast<const long long*>(r), er,
+                  *reinterpret_cast<const long long*>(s), es, tT.k);
+    else
+      *t = value(t, E) + (value(r, er) + value(s, es));
+  }
+}
+
 // Registers: the kernel waits on memory, shared memory and dependent integer operations in turn, so
 // resident warps are worth more than registers up to the point where lines spill.
 template <int N>
@@ -236,36 +272,17 @@ __global__ void __maxnreg__(ax_fx_regs<N>())
   *ax_line_scale<N>(U, 1, i, j) = Er;
   *ax_line_scale<N>(U, 2, i, j) = Es;
   const bool slow = __syncthreads_or(max(Er, Es) == FX_NO_SCALE);
-  // t-lines; the three parts are added on the largest of their scales (what a smaller one loses there is
-  // below 2^-60 of the sum's largest part) and rounded to double once
+  // t-lines, and the three parts added
   {
     int h[N], l[N], E;
     const bool scaled = fx_split_line<N>(U + col, PL, h, l, E);
-    auto sum = [&](int q, long long r, int er, int es) {
-      const int m = max(E, max(er, es));
-      r = fx_shr(r, m - E) + fx_shr(reinterpret_cast<const long long*>(R)[col + PL * q], m - er) +
-          fx_shr(reinterpret_cast<const long long*>(S)[col + PL * q], m - es);
-      return fx_double(r, m - tT.k);
-    };
     if (scaled && !slow) {
       fx_contract<N, N, -1>(tT, h, l, [&](int q, long long r) {
-        U[col + PL * q] = sum(q, r, *ax_line_scale<N>(U, 1, j, q), *ax_line_scale<N>(U, 2, i, q));
+        U[col + PL * q] = ax_sum(r, E, reinterpret_cast<const long long*>(R)[col + PL * q], *ax_line_scale<N>(U, 1, j, q),
+                                 reinterpret_cast<const long long*>(S)[col + PL * q], *ax_line_scale<N>(U, 2, i, q), tT.k);
       });
     } else {
-      if (scaled)
-        fx_contract<N, N, -1>(tT, h, l, [&](int q, long long r) { reinterpret_cast<long long*>(U)[col + PL * q] = r; });
-      else
-        ax_slow_line<N>(a.D, true, U + col, U + col, PL);
-      auto value = [&](const double* p, int e) {
-        return e == FX_NO_SCALE ? *p : fx_double(*reinterpret_cast<const long long*>(p), e - tT.k);
-      };
-#pragma unroll 1
-      for (int q = 0; q < N; ++q) {
-        const int er = *ax_line_scale<N>(U, 1, j, q), es = *ax_line_scale<N>(U, 2, i, q);
-        double* u = U + col + PL * q;
-        if (scaled && max(er, es) != FX_NO_SCALE) *u = sum(q, *reinterpret_cast<const long long*>(u), er, es);
-        else *u = value(u, scaled ? E : FX_NO_SCALE) + (value(R + col + PL * q, er) + value(S + col + PL * q, es));
-      }
+      ax_slow_column<N>(a.D, tT, U, i, j);
     }
   }
   // U: A_L u, each thread's own column

@@ -16,7 +16,7 @@
 //
 // Measured on GB300 (us per launch; in brackets the FP64 kernel this one replaced, at 91% of the FP64
 // pipe): 24^3 elements p = 7 377 [1190], p = 5 158 [460], p = 3 59 [150]; 16^3 p = 9 236 [700].  The
-// multiply-adds keep their pipe (32 lanes/clk/SM) about 68% busy; a result's two sums in a row beat all results' sums
+// multiply-adds keep their pipe (32 lanes/clk/SM) 64% busy; a result's two sums in a row beat all results' sums
 // input by input (more chains in flight, 500 instead of 406 at p = 7: the accumulator stays in the
 // pipe), and 64 registers beat 80 and 96 (440).
 //
