@@ -55,8 +55,8 @@ enum { SE_BC_DIRICHLET = 0, SE_BC_NEUMANN = 1 };
  * The FP64 kernels contract lines in fixed point.  Operator and transfers: every line on the scale of its
  * own largest value, 2-norm error 0.3 to 1.0 of that of FP64 dot products (1.19 for the pair of orders 2, 1).
  * Schwarz solves: every window on the scale of its largest residual, error 0.3 to 0.7 of the FP64
- * solve's for random and smooth residuals, up to 1.5 around a residual 10^8 times its neighbours.  What cannot
- * share a scale (infinities, NaN, magnitudes near the ends of the range) is computed in FP64. */
+ * solve's, up to 1.0 around a residual 10^8 times its neighbours.  What cannot share a scale (infinities,
+ * NaN, magnitudes near the ends of the range) is computed in FP64. */
 enum { SE_FP64 = 0, SE_FP32 = 1, SE_DF64 = 2 };
 enum { SE_SMOOTH_JACOBI = 0, SE_SMOOTH_RAS = 1, SE_SMOOTH_ASM = 2 };
 enum { SE_FPCG = 0, SE_FGMRES = 1 };
